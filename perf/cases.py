@@ -79,7 +79,9 @@ def draw(rng):
     if kind == "step":
         solver = rng.choice(("ptc", "nk"))
         most = 7 if solver == "ptc" else 56
-        return dict(kind=kind, flow="vortex", a=_log(rng, 4, most), b=_log(rng, 4, most), c=0,
+        a = _log(rng, 4, most)
+        b = min(most, max(4, int(a * rng.uniform(0.6, 1.5))))   # elements of moderate aspect ratio
+        return dict(kind=kind, flow="vortex", a=a, b=b, c=0,
                     levels=rng.choice(("2-1-0", "3-2-1-0") if solver == "nk" else ("2-1-0",)),
                     blocks=rng.choice(("fp32", "bf16") if solver == "ptc" else ("fp32", "fp32", "fp64")), flux="dw",
                     solver=solver, curved=False)
