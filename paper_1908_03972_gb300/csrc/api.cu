@@ -505,20 +505,6 @@ static pmg_status check_level(const Ctx& c, int level) {
   return PMG_OK;
 }
 
-// Levels whose blocks not even a cluster of 8 CTAs can hold in shared memory
-// (n above about 470 in FP64) have a residual but no smoother.
-static pmg_status check_factorable(const Ctx& c, int level) {
-  const int lim = factor_max_n(c.cfg.block_prec);
-  for (int l = 0; l < c.cfg.n_levels; ++l) {
-    if (level >= 0 && l != level) continue;
-    if (c.lev[l].n > lim)
-      return fail(PMG_EINVAL, "element blocks of level " + std::to_string(l) + " (n = " + std::to_string(c.lev[l].n) +
-                                  ") exceed the shared-memory factorisation (n <= " + std::to_string(lim) +
-                                  " in this block precision)");
-  }
-  return PMG_OK;
-}
-
 static cudaError_t copy_in(const Ctx& c, double* dst, const double* src, size_t count, int on_device) {
   return cudaMemcpyAsync(dst, src, count * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                          c.stream);
@@ -1252,10 +1238,6 @@ static pmg_status nk_stage_solve(Ctx& c, int* iters, double* drop, int* n_refres
 }
 
 static pmg_status stage_solve(Ctx& c, int* iters, double* drop, int* n_refresh, int* vcycles = nullptr) {
-  {
-    pmg_status fs = check_factorable(c, -1);
-    if (fs) return fs;
-  }
   if (c.stage_solver == PMG_STAGE_NK) return nk_stage_solve(c, iters, drop, n_refresh, vcycles);
   if (vcycles) *vcycles = -1;   // the caller counts pseudo-iterations
   if (!c.F0_valid) {
@@ -1626,10 +1608,6 @@ pmg_status pmg_factor_blocks(pmg_ctx* h, int level) {
   Ctx& c = h->c;
   if (!c.mesh_ready) return fail(PMG_ESTATE, "mesh not uploaded");
   if (level < -1 || level >= c.cfg.n_levels) return fail(PMG_EINVAL, "level out of range");
-  {
-    pmg_status fs = check_factorable(c, level);
-    if (fs) return fs;
-  }
   for (int l = 0; l < c.cfg.n_levels; ++l) {
     if (level >= 0 && l != level) continue;
     if (!c.lev[l].assembled) return fail(PMG_ESTATE, "blocks not assembled");
@@ -1711,10 +1689,6 @@ pmg_status pmg_vcycle(pmg_ctx* h, double dtau, int refresh, double* res_norm_out
   if (!c.mesh_ready) return fail(PMG_ESTATE, "mesh not uploaded");
   if (!c.stage_ready) return fail(PMG_ESTATE, "stage data not set");
   if (!(dtau > 0.0)) return fail(PMG_EINVAL, "dtau must be positive");
-  {
-    pmg_status fs = check_factorable(c, -1);
-    if (fs) return fs;
-  }
   if (!refresh)
     for (int l = 0; l < c.cfg.n_levels; ++l)
       if (!c.lev[l].factored) return fail(PMG_ESTATE, "smoother not built: call with refresh = 1 first");

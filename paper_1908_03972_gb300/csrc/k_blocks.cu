@@ -8,14 +8,14 @@
 //    numbers pushed through the same flux code as the residual; the FR
 //    structure (derivative, extrapolation, correction) is applied in
 //    tensor-product form.  Neighbour states are frozen.
-//  * factor: one CTA per element equilibrates the block with power-of-two
-//    row and column scales (exact in any precision) and inverts it by
-//    Gauss-Jordan elimination with partial pivoting in the working precision
-//    (FP64, or FP32 for the mixed-precision smoother).  The explicit inverse
-//    turns every smoothing sweep into a batched matrix-vector product.  The
-//    equilibrated rows have unit size, so a pivot that is not finite or not
-//    above n eps of the working precision (the rounding a dependent row leaves
-//    after elimination) marks a block that is singular to that precision: the
+//  * factor (k_factor.cu): the block equilibrated with power-of-two row and
+//    column scales (exact in any precision) and inverted by Gauss-Jordan
+//    elimination with partial pivoting in the working precision (FP64, or FP32
+//    for the mixed-precision smoother).  The explicit inverse turns every
+//    smoothing sweep into a batched matrix-vector product.  The equilibrated
+//    rows have unit size, so a pivot that is not finite or not above n eps of
+//    the working precision (the rounding a dependent row leaves after
+//    elimination) marks a block that is singular to that precision: the
 //    element is flagged for the host (PMG_ESINGULAR).
 //  * apply: x = cs .* (inv(D^) (rs .* r)); each thread owns four consecutive
 //    rows and streams the column-major inverse with 16-byte (FP32) or
@@ -152,186 +152,6 @@ void launch_assemble(const Ctx& c, const LevelDev& L, const double* q, const dou
   }
 #undef PMG_ASM
   if (c.ph.mu > 0.0) launch_assemble_visc(c, L, q, s);
-}
-
-// -------------------------------------------------------------------- factor
-__device__ __forceinline__ double pow2_inv_scale(double m) {
-  // 2^-k with m * 2^-k in [0.5, 1); 1 for m == 0
-  if (!(m > 0.0)) return 1.0;
-  int ex;
-  frexp(m, &ex);
-  return ldexp(1.0, -ex);
-}
-
-// Machine epsilon of the working precision; the smallest pivot magnitude
-// accepted is n eps (the equilibrated rows have unit size).
-template <class W> struct Eps;
-template <> struct Eps<float> { static constexpr double value = 1.1920928955078125e-07; };
-template <> struct Eps<double> { static constexpr double value = 2.220446049250313e-16; };
-
-template <class W>
-__global__ void __launch_bounds__(256) factor_kernel(int n, const double* __restrict__ Din, W* __restrict__ Dinv,
-                                                     double* __restrict__ rs, double* __restrict__ cs,
-                                                     int* __restrict__ flag, int flag_base) {
-  using T = typename Blk<W>::acc;   // elimination arithmetic (FP32 for BF16 storage)
-  extern __shared__ unsigned char smem_raw[];
-  T* A = reinterpret_cast<T*>(smem_raw);                       // n * n, row-major
-  T* colk = A + n * n;                                          // n
-  int* perm = reinterpret_cast<int*>(colk + n);                 // n
-  double* sr = reinterpret_cast<double*>(((uintptr_t)(perm + n) + 7) & ~(uintptr_t)7);   // n
-  double* sc = sr + n;                                          // n
-  __shared__ int s_piv;
-  __shared__ int s_bad;
-  const int e = blockIdx.x;
-  const double* D = Din + (size_t)e * n * n;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  if (tid == 0) s_bad = 0;
-  // row scales
-  for (int i = tid; i < n; i += nt) {
-    double m = 0.0;
-    for (int j = 0; j < n; ++j) m = fmax(m, fabs(D[(size_t)i * n + j]));
-    sr[i] = pow2_inv_scale(m);
-  }
-  __syncthreads();
-  for (int j = tid; j < n; j += nt) {
-    double m = 0.0;
-    for (int i = 0; i < n; ++i) m = fmax(m, fabs(D[(size_t)i * n + j] * sr[i]));
-    sc[j] = pow2_inv_scale(m);
-  }
-  __syncthreads();
-  for (int t = tid; t < n * n; t += nt) {
-    int i = t / n, j = t - i * n;
-    A[t] = (T)(D[t] * sr[i] * sc[j]);
-  }
-  __syncthreads();
-  // Gauss-Jordan with partial pivoting, in place
-  for (int k = 0; k < n; ++k) {
-    if (tid < 32) {
-      double best = -1.0;
-      int bi = k;
-      for (int i = k + tid; i < n; i += 32) {
-        double a = fabs((double)A[i * n + k]);
-        if (a > best) { best = a; bi = i; }
-      }
-      for (int off = 16; off > 0; off >>= 1) {
-        double ob = __shfl_down_sync(0xffffffffu, best, off);
-        int oi = __shfl_down_sync(0xffffffffu, bi, off);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (tid == 0) {
-        s_piv = bi;
-        perm[k] = bi;
-        if (!(best > n * Eps<T>::value) || isinf(best)) s_bad = 1;
-      }
-    }
-    __syncthreads();
-    const int p = s_piv;
-    if (p != k)
-      for (int j = tid; j < n; j += nt) { T t = A[k * n + j]; A[k * n + j] = A[p * n + j]; A[p * n + j] = t; }
-    __syncthreads();
-    T piv = A[k * n + k];
-    T ipiv = (T)1 / piv;
-    __syncthreads();
-    for (int j = tid; j < n; j += nt) A[k * n + j] = (j == k) ? ipiv : A[k * n + j] * ipiv;
-    for (int i = tid; i < n; i += nt) colk[i] = A[i * n + k];
-    __syncthreads();
-    if (sizeof(T) == 4 && n <= nt) {
-      // FP32 elimination (issue-bound): thread (r0, j) updates column j in
-      // rows r0, r0 + rpp, ... with the pivot row's entry in a register and
-      // no index division; the same operation on every entry as below
-      const int rpp = nt / n, j = tid % n, r0 = tid / n;
-      if (r0 < rpp) {
-        const T akj = A[k * n + j];
-        for (int i = r0; i < n; i += rpp) {
-          if (i == k) continue;
-          const T f = colk[i];
-          if (j == k) A[i * n + j] = -f * akj;
-          else A[i * n + j] -= f * akj;
-        }
-      }
-    } else {
-      for (int t = tid; t < n * n; t += nt) {
-        int i = t / n, j = t - i * n;
-        if (i == k) continue;
-        T f = colk[i];
-        if (j == k) A[t] = -f * A[k * n + k];
-        else A[t] -= f * A[k * n + j];
-      }
-    }
-    __syncthreads();
-  }
-  // undo the row interchanges as column interchanges, last first
-  for (int k = n - 1; k >= 0; --k) {
-    int p = perm[k];
-    if (p != k)
-      for (int i = tid; i < n; i += nt) { T t = A[i * n + k]; A[i * n + k] = A[i * n + p]; A[i * n + p] = t; }
-    __syncthreads();
-  }
-  // store column-major: Dinv[e][col][row]
-  W* out = Dinv + (size_t)e * n * n;
-  for (int t = tid; t < n * n; t += nt) {
-    int col = t / n, row = t - col * n;
-    out[t] = (W)A[row * n + col];
-  }
-  for (int i = tid; i < n; i += nt) {
-    rs[(size_t)e * n + i] = sr[i];
-    cs[(size_t)e * n + i] = sc[i];
-  }
-  if (tid == 0 && s_bad) atomicMax(flag, flag_base + e + 1);
-}
-
-static size_t factor_smem(int n, int wbytes) {
-  size_t b = (size_t)n * n * wbytes + (size_t)n * wbytes + (size_t)n * 4;
-  b = (b + 7) & ~(size_t)7;
-  return b + 2 * (size_t)n * 8;
-}
-
-void launch_factor(const Ctx& c, LevelDev& L, int level, int prec, int* flag, cudaStream_t s) {
-  const int n = L.n, base = level * c.E;   // the flag holds 1 + level E + element of the highest bad block
-  const int C = factor_cluster_size(n, prec);
-  if (C > 1) {   // too large for one CTA: a cluster of C (k_factor_cluster.cu)
-    launch_factor_cluster(c, L, level, prec, C, flag, s);
-    return;
-  }
-  if (prec == PMG_PREC_FP64)
-    factor_kernel<double><<<c.E, 256, factor_smem(n, 8), s>>>(n, L.Dfull, (double*)L.Dinv, L.rs, L.cs, flag, base);
-  else if (prec == PMG_PREC_BF16R)
-    factor_kernel<__nv_bfloat16><<<c.E, 256, factor_smem(n, 4), s>>>(n, L.Dfull, (__nv_bfloat16*)L.Dinv, L.rs,
-                                                                       L.cs, flag, base);
-  else
-    factor_kernel<float><<<c.E, 256, factor_smem(n, 4), s>>>(n, L.Dfull, (float*)L.Dinv, L.rs, L.cs, flag, base);
-}
-
-// Largest block the shared-memory factorisation holds in the precision prec:
-// one CTA (227 KB) up to n = 168 in FP64 and 238 in FP32 and BF16 (their
-// elimination runs in FP32), a cluster of up to 8 CTAs beyond.
-int factor_max_n(int prec) {
-  int n = 4;
-  while (factor_cluster_size(n + 1, prec) > 0) ++n;
-  return n;
-}
-
-// Opt the factor kernels into the dynamic shared memory the largest block
-// needs (done once, outside any stream capture).  Levels whose blocks exceed
-// factor_max_n are left out; the calls that would factor them fail first.
-cudaError_t prepare_kernels(const Ctx& c) {
-  int nmax = 4;
-  for (int l = 0; l < c.cfg.n_levels; ++l) {
-    const int C = factor_cluster_size(c.lev[l].n, c.cfg.block_prec);
-    if (C == 1) nmax = std::max(nmax, c.lev[l].n);
-    if (C > 1) {
-      cudaError_t e = prepare_factor_cluster(c.lev[l].n, c.cfg.block_prec, C);
-      if (e != cudaSuccess) return e;
-    }
-  }
-  cudaError_t e = cudaFuncSetAttribute(factor_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)factor_smem(nmax, 8));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(factor_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)factor_smem(nmax, 4));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(factor_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)factor_smem(nmax, 4));
 }
 
 // --------------------------------------------------------------------- apply

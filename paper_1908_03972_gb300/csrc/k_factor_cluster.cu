@@ -1,19 +1,20 @@
-// k_factor_cluster.cu -- the element-block factorisation of k_blocks.cu
-// (Section 2.4: the smoother's blocks D_e, power-of-two equilibration, then
-// Gauss-Jordan elimination with partial pivoting to the explicit inverse) for
-// blocks too large for one CTA's shared memory: hexahedra at P = 3 have
-// n = 5 (P+1)^3 = 320, 400 KB in FP32.
+// k_factor_cluster.cu -- the element-block factorisation (Section 2.4: the
+// smoother's blocks D_e, power-of-two equilibration, then Gauss-Jordan
+// elimination with partial pivoting to the explicit inverse) column by column
+// in the shared memory of a thread-block cluster.  The solver factors with
+// k_factor.cu; this kernel, chosen by PMG_FACTOR_CLUSTER, states the same
+// elimination one pivot at a time, and the tests hold the other to its result
+// bit for bit.
 //
-// A thread-block cluster of C CTAs (2, 4 or 8) owns one block.  CTA r keeps
+// A cluster of C CTAs (2, 4 or 8) owns one block.  CTA r keeps
 // columns [r nc, (r+1) nc) of the equilibrated matrix in its shared memory
 // (nc = ceil(n / C)); every step k of the elimination needs from the rest of
 // the cluster only the pivot row index and the pivot column, which the CTA
 // owning column k publishes in its shared memory and the others read through
 // distributed shared memory, between two cluster barriers.  Row interchanges
-// and the updates of each CTA's columns are local.  The operations on every
-// entry are those of the one-CTA kernel in the same order, so both give the
-// same inverse bit for bit.  The final column interchanges (the row
-// interchanges undone) become a permutation of the stored columns.
+// and the updates of each CTA's columns are local.  The final column
+// interchanges (the row interchanges undone) become a permutation of the
+// stored columns.
 #include <cooperative_groups.h>
 
 #include "pmg_internal.h"
@@ -25,7 +26,7 @@ namespace pmg {
 namespace {
 
 __device__ __forceinline__ double pow2_inv_scale_c(double m) {
-  // 2^-k with m * 2^-k in [0.5, 1); 1 for m == 0 (as in the one-CTA kernel)
+  // 2^-k with m * 2^-k in [0.5, 1); 1 for m == 0
   if (!(m > 0.0)) return 1.0;
   int ex;
   frexp(m, &ex);
@@ -139,8 +140,7 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kClusterThreads)
     for (int jl = tid; jl < m; jl += nt)
       A[(size_t)k * nc + jl] = (c0 + jl == k) ? ipiv : A[(size_t)k * nc + jl] * ipiv;
     __syncthreads();
-    // The update of the own columns; every entry sees the same operation as
-    // in the one-CTA kernel.  FP32 elimination (issue-bound): thread (r0, jl)
+    // The update of the own columns.  FP32 elimination (issue-bound): thread (r0, jl)
     // updates column jl in rows r0, r0 + rpp, ... (rpp = nt / m rows per
     // pass), the pivot row's entry in a register and no index divided in the
     // loop -- 1.57x faster on n = 320.  FP64 elimination (bound by the FP64
@@ -199,12 +199,6 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kClusterThreads)
 
 namespace {
 
-size_t one_cta_smem(int n, int tbytes) {   // the k_blocks.cu kernel's layout
-  size_t b = (size_t)n * n * tbytes + (size_t)n * tbytes + (size_t)n * 4;
-  b = (b + 7) & ~(size_t)7;
-  return b + 2 * (size_t)n * 8;
-}
-
 constexpr size_t kSmemBudget = (size_t)227 * 1024 - 64;   // dynamic bytes a CTA may take
 
 template <class W>
@@ -225,18 +219,13 @@ cudaError_t prepare_w(int C, size_t bytes) {
 
 }  // namespace
 
-// CTAs per block: 1 (the one-CTA kernel of k_blocks.cu), 2, 4 or 8 (a
-// cluster), 0 when even 8 CTAs cannot hold it.  PMG_FACTOR_CLUSTER = 2, 4 or 8
-// puts every block that such a cluster holds on the cluster kernel (tests).
+// CTAs per block when PMG_FACTOR_CLUSTER = 2, 4 or 8 asks for this kernel and
+// such a cluster holds the block, else 0 (the register kernel of k_factor.cu).
 int factor_cluster_size(int n, int prec) {
   const int tb = prec == PMG_PREC_FP64 ? 8 : 4;
   int force = 0;
   if (const char* env = getenv("PMG_FACTOR_CLUSTER")) force = atoi(env);
-  if ((force == 2 || force == 4 || force == 8) && factor_cluster_smem(n, force, tb) <= kSmemBudget) return force;
-  if (one_cta_smem(n, tb) <= (size_t)227 * 1024) return 1;
-  for (int C : {2, 4, 8})
-    if (factor_cluster_smem(n, C, tb) <= kSmemBudget) return C;
-  return 0;
+  return (force == 2 || force == 4 || force == 8) && factor_cluster_smem(n, force, tb) <= kSmemBudget ? force : 0;
 }
 
 void launch_factor_cluster(const Ctx& c, LevelDev& L, int level, int prec, int C, int* flag, cudaStream_t s) {
