@@ -214,6 +214,7 @@ pmg_status pmg_create(const pmg_config* cfg, void* stream, pmg_ctx** out) {
   c.ph.p_ref = cfg->p_gauge;
   c.ph.inv_gamma = 1.0 / cfg->gamma;
   c.ph.inv_gm1 = 1.0 / (cfg->gamma - 1.0);
+  c.ph.inv_Cp = (cfg->gamma - 1.0) / cfg->gamma;
   c.ph.mu = cfg->mu;
   c.ph.kT = cfg->mu > 0.0 ? cfg->mu * c.ph.Cp / cfg->Pr : 0.0;
   for (int v = 0; v < 5; ++v) { c.ph.nw[v] = 1.0; c.ph.qinf[v] = 0.0; }
@@ -400,12 +401,25 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
       for (int k = 0; k < L.n1; ++k) L.op.D[i][k] = r.D[i * L.n1 + k];
       L.op.lm[i] = r.lm[i]; L.op.lp[i] = r.lp[i]; L.op.gL[i] = r.gL[i]; L.op.gR[i] = r.gR[i];
     }
+    // D - gL lm^T - gR lp^T: the derivative with the extrapolated part of both
+    // faces' corrections folded in, so that the divergence of a line is
+    // Dt F + gL (common flux at -1) + gR (common flux at +1)
+    for (int i = 0; i < L.n1; ++i)
+      for (int k = 0; k < L.n1; ++k) {
+        L.op.Dt[i][k] = (double)((long double)r.D[i * L.n1 + k] - (long double)r.gL[i] * r.lm[k] -
+                                 (long double)r.gR[i] * r.lp[k]);
+        L.op.hlm[k] = 0.5 * r.lm[k];
+        L.op.hlp[k] = 0.5 * r.lp[k];
+      }
     // BR2 lifting factor: penalty eta_f = 4 (faces of a quadrilateral) times
     // the DG correction's g_R'(1) = (P+1)^2 / 2
     L.op.pen = 4.0 * 0.5 * L.n1 * L.n1;
     memset(&L.opw, 0, sizeof(L.opw));
     for (int i = 0; i < L.n1; ++i) {
-      for (int k = 0; k < L.n1; ++k) L.opw.D[i][k] = dw_const(L.op.D[i][k]);
+      for (int k = 0; k < L.n1; ++k) {
+        L.opw.D[i][k] = dw_const(L.op.D[i][k]);
+        L.opw.Dt[i][k] = dw_const(L.op.Dt[i][k]);
+      }
       L.opw.lm[i] = dw_const(L.op.lm[i]);
       L.opw.lp[i] = dw_const(L.op.lp[i]);
       L.opw.gL[i] = dw_const(L.op.gL[i]);
@@ -451,6 +465,8 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
       const size_t nj = c.dim == 3 ? (size_t)4 * c.E * 6 * L.NF : (size_t)3 * c.E * 4 * L.n1;
       if (dalloc(&L.Gb, ng) || dalloc(&L.Qj, nj) || dalloc(&L.fJinv, geo[l].fJinv.size()))
         return fail(PMG_ENOMEM, "device allocation failed for level data");
+      // the gradient launch leaves out P = 0, where the broken gradient is zero
+      PMG_CK(cudaMemset(L.Gb, 0, ng * 8));
       PMG_CK(cudaMemcpy(L.fJinv, geo[l].fJinv.data(), geo[l].fJinv.size() * 8, cudaMemcpyHostToDevice));
     }
     PMG_CK(cudaMemset(L.S, 0, L.tot * 8));

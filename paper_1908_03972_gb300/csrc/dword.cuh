@@ -25,7 +25,7 @@
 
 namespace pmg {
 
-struct dw {
+struct alignas(8) dw {   // one 8-byte access
   float h, l;
 };
 

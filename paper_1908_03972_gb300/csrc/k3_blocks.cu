@@ -178,6 +178,7 @@ __global__ void __launch_bounds__(64) apply3_kernel(int E, const W* __restrict__
   if (!active) return;
   Acc acc[5] = {0, 0, 0, 0, 0};
   const W* Dm = Dinv + (size_t)e * n * n + pt;
+#pragma unroll 10
   for (int k = 0; k < n; ++k) {
     const Acc rk = sr[le][k];
 #pragma unroll

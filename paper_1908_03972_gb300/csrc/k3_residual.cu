@@ -10,11 +10,24 @@
 //    faces take the ghost state of their type.
 //  * volume3: one thread per solution point, EPB3 elements per CTA.  The
 //    contravariant fluxes F^i = f . J a^i of the element's points go to
-//    shared memory; the face jumps (common flux in the reference direction
-//    minus the extrapolated flux polynomial), the Lagrange derivative along
-//    the three directions and the DG correction follow, then the epilogue of
-//    the requested mode, a deterministic per-CTA sum of squares for the norm,
-//    and with APPLY the element-Jacobi update q += cs .* D^-1 (rs .* (F - S)).
+//    shared memory, the common fluxes of its faces by asynchronous copies; a
+//    line's divergence is Dt F + gL F_com(-1) + gR F_com(+1), the derivative
+//    with the extrapolated part of the correction folded in (OpTab::Dt), then
+//    the epilogue of the requested mode, a deterministic per-CTA sum of squares
+//    for the norm, and with APPLY the element-Jacobi update
+//    q += cs .* D^-1 (rs .* (F - S)).
+//
+// All three kernels are bound by FP64 issue: a warp instruction takes 64 cycles
+// of its sub-partition however many lanes are active, so what counts is FP64
+// instructions per warp.  The face jumps are not formed (one extrapolation per
+// face point and equation less), the corrected gradient adds only the face
+// corrections to the broken gradient the gradient launch wrote (12 planes read
+// instead of 36 derivative sums recomputed: 96 bytes against about 100 FP64
+// instructions a point), the viscous and inviscid fluxes are joined as
+// symmetric Cartesian tensors before the metric terms contract them, and the
+// gradient launch subtracts one reference per element, once per value.
+// Measured on 3,072 viscous hexahedra at P = 3 (one GB300): gradient 57 -> 38
+// us, face flux 136 -> 114 us, residual 165 -> 108 us.
 //
 // Layout: states q[(v*E + e)*N + pt], v < 5, pt = (k*(P+1) + j)*(P+1) + i;
 // metric planes met[c*E*N + e*N + pt], c = 3 i + n for J a^i_n, c = 9 for 1/J;
@@ -128,52 +141,59 @@ __global__ void __launch_bounds__(64) face_flux3_kernel(const int* __restrict__ 
   qm[0] += ph.p_ref;
   qp[0] += ph.p_ref;
   double out[5];
-  roe3_flux_jump(qm, qp, dq, pgm, pgp, nrm, dS, ph, out);
+  roe_jump_d<3>(qm, qp, dq, pgm, pgp, nrm, dS, ph, out);
   const size_t fplane = (size_t)E * 6 * NF;
   const size_t iL = ((size_t)eL * 6 + fL) * NF + fp;
   if (VISC) {
-    double gm[12], gp[12];
-    const double* bL = Gb + (size_t)eL * N;
-#pragma unroll
-    for (int c = 0; c < 12; ++c) {
-      double t = 0.0;
-#pragma unroll
-      for (int m = 0; m < n1; ++m)
-        t = fma((fL & 1) ? lp[m] : lm[m], __ldg(bL + c * plane + line_pt3<P>(fL, a, b, m)), t);
-      gm[c] = t;
-      gp[c] = t;
-    }
-    double iJp = __ldg(fJinv + iL);
-    const double iJm = iJp;
-    if (!bnd) {
-      const int a2 = fp2 % n1, b2 = fp2 / n1;
-      const double* bR = Gb + (size_t)eR * N;
-#pragma unroll
-      for (int c = 0; c < 12; ++c) {
-        double t = 0.0;
-#pragma unroll
-        for (int m = 0; m < n1; ++m)
-          t = fma((fR & 1) ? lp[m] : lm[m], __ldg(bR + c * plane + line_pt3<P>(fR, a2, b2, m)), t);
-        gp[c] = t;
-      }
-      iJp = __ldg(fJinv + ((size_t)eR * 6 + fR) * NF + fp2);
-    }
+    // mean of both sides' broken-gradient traces (a boundary mirrors the
+    // element), plus the lifting; at P = 0 the broken gradient is zero
+    const double iJm = __ldg(fJinv + iL);
+    const double iJp = bnd ? iJm : __ldg(fJinv + ((size_t)eR * 6 + fR) * NF + fp2);
     const double wl = 0.25 * op.pen * (iJm + iJp) * dS;
-    double gc[12], fv[12];
+    double gc[12];
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
-      for (int k = 0; k < 4; ++k) gc[c * 4 + k] = fma(wl * nrm[c], dq[k + 1], 0.5 * (gm[c * 4 + k] + gp[c * 4 + k]));
-    const double uc[3] = {0.5 * (qm[1] + qp[1]), 0.5 * (qm[2] + qp[2]), 0.5 * (qm[3] + qp[3])};
-    viscous_flux3(uc, gc, ph, fv);
-    const int nr = (bnd && fR != PMG_BC_FARFIELD) ? 3 : 4;   // walls: no viscous energy flux
+      for (int k = 0; k < 4; ++k) gc[c * 4 + k] = (wl * nrm[c]) * dq[k + 1];
+    if (P > 0) {
+      const int a2 = fp2 % n1, b2 = fp2 / n1;
+      const double* bL = Gb + (size_t)eL * N;
+      const double* bR = Gb + (size_t)(bnd ? eL : eR) * N;
+      const int fo = bnd ? fL : fR, ao = bnd ? a : a2, bo = bnd ? b : b2;
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
-      if (r < nr) out[r + 1] -= (fv[r] * nrm[0] + fv[4 + r] * nrm[1] + fv[8 + r] * nrm[2]) * dS;
+      for (int m = 0; m < n1; ++m) {
+        const double wL = (fL & 1) ? op.hlp[m] : op.hlm[m], wR = (fo & 1) ? op.hlp[m] : op.hlm[m];
+        const int iLp = line_pt3<P>(fL, a, b, m), iRp = line_pt3<P>(fo, ao, bo, m);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+          gc[c] = fma(wL, __ldg(bL + c * plane + iLp), gc[c]);
+          gc[c] = fma(wR, __ldg(bR + c * plane + iRp), gc[c]);
+        }
+      }
+    }
+    // viscous flux through n dS at q_com: mu (g + g^T) n - 2/3 mu div n, and
+    // its work on u_com plus the heat flux
+    const double mdS = ph.mu * dS, kdS = ph.kT * dS;
+    const double d23 = (gc[0] + gc[5] + gc[10]) * (2.0 / 3.0);
+    const double s01 = gc[1] + gc[4], s02 = gc[2] + gc[8], s12 = gc[6] + gc[9];
+    double t[3];
+    t[0] = fma(2.0 * gc[0] - d23, nrm[0], fma(s01, nrm[1], s02 * nrm[2]));
+    t[1] = fma(2.0 * gc[5] - d23, nrm[1], fma(s01, nrm[0], s12 * nrm[2]));
+    t[2] = fma(2.0 * gc[10] - d23, nrm[2], fma(s02, nrm[0], s12 * nrm[1]));
+    double wk = 0.0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      out[1 + c] = fma(-mdS, t[c], out[1 + c]);
+      wk = fma(fma(0.5, dq[1 + c], qm[1 + c]), t[c], wk);
+    }
+    const bool wall = bnd && fR != PMG_BC_FARFIELD;   // walls: no viscous energy flux
+    const double ht = fma(gc[3], nrm[0], fma(gc[7], nrm[1], gc[11] * nrm[2]));
+    if (!wall) out[4] = fma(-mdS, wk, fma(-kdS, ht, out[4]));
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      Qj[k * fplane + iL] = 0.5 * dq[k + 1];
-      if (!bnd) Qj[k * fplane + ((size_t)eR * 6 + fR) * NF + fp2] = -0.5 * dq[k + 1];
+      const double hj = 0.5 * dq[k + 1];
+      Qj[k * fplane + iL] = hj;
+      if (!bnd) Qj[k * fplane + ((size_t)eR * 6 + fR) * NF + fp2] = -hj;
     }
   }
 #pragma unroll
@@ -185,14 +205,22 @@ __global__ void __launch_bounds__(64) face_flux3_kernel(const int* __restrict__ 
   }
 }
 
+// One double by an asynchronous copy (8 bytes: the only alignment every
+// caller's buffers have).
+__device__ __forceinline__ void async_g2s(double* dst, const double* src) {
+  const unsigned int d = (unsigned int)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // With VISC the contravariant fluxes take f_inv - f_vis: the viscous flux at
-// each solution point from the corrected gradient, the reference derivatives
-// of (u, v, w, T) plus the DG correction of the face jumps Qj on the two faces
-// of each line through the point (eq. com_q), then the chain rule with the
-// metric terms.
+// each solution point from the corrected gradient, the broken gradient Gb plus
+// the DG correction of the face jumps Qj on the two faces of each line through
+// the point (eq. com_q), chain rule with the metric terms.
 template <int P, class W, bool APPLY, bool VISC>
 __global__ void __launch_bounds__(64) volume3_kernel(int E, const double* q, const double* __restrict__ met,
                                                      const double* __restrict__ Fcom, const double* __restrict__ Qj,
+                                                     const double* __restrict__ Gb,
                                                      OpTab op, Phys ph,
                                                      double* __restrict__ out, int mode, double inv_odt,
                                                      const double* __restrict__ src, const double* __restrict__ S,
@@ -203,97 +231,121 @@ __global__ void __launch_bounds__(64) volume3_kernel(int E, const double* q, con
   constexpr int n1 = P + 1, N = n1 * n1 * n1, NF = n1 * n1, EPB = EPB3<P>::value, n = 5 * N;
   using Acc = typename Blk<W>::acc;
   __shared__ double sF[EPB][3][5][N];
-  __shared__ double sJ[EPB][6][5][NF];
+  __shared__ double sC[5][EPB * 6 * NF];                        // common fluxes, outward
+  __shared__ double sQ[VISC ? 4 : 1][VISC ? EPB * 6 * NF : 1];  // face jumps
   __shared__ Acc sr[APPLY ? EPB : 1][APPLY ? n : 1];
-  __shared__ double sD[n1][n1], sgL[n1], sgR[n1], slm[n1], slp[n1];
+  __shared__ double sD[n1][n1], sgL[n1], sgR[n1];
   __shared__ double sred[2];
-  __shared__ double sV[VISC ? EPB : 1][4][VISC ? N : 1];   // u, v, w, T of the element
   const int le = threadIdx.x / N, pt = threadIdx.x - le * N;
   const int e = blockIdx.x * EPB + le;
   const bool active = (le < EPB) && (e < E);
   const size_t plane = (size_t)E * N;
   const size_t fplane = (size_t)E * 6 * NF;
-  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = op.D[threadIdx.x / n1][threadIdx.x % n1];
+  {
+    const int e0 = blockIdx.x * EPB, nf = min(EPB, E - e0) * 6 * NF;
+    const size_t f0 = (size_t)e0 * 6 * NF;
+    for (int t = threadIdx.x; t < nf; t += blockDim.x) {
+      if (VISC)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) async_g2s(&sQ[VISC ? k : 0][VISC ? t : 0], Qj + k * fplane + f0 + t);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) async_g2s(&sC[v][t], Fcom + v * fplane + f0 + t);
+    }
+  }
+  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = op.Dt[threadIdx.x / n1][threadIdx.x % n1];
   if (threadIdx.x < n1) {
     sgL[threadIdx.x] = op.gL[threadIdx.x];
     sgR[threadIdx.x] = op.gR[threadIdx.x];
-    slm[threadIdx.x] = op.lm[threadIdx.x];
-    slp[threadIdx.x] = op.lp[threadIdx.x];
   }
   const size_t gi = (size_t)e * N + pt;
+  const int i = pt % n1, j = (pt / n1) % n1, k = pt / (n1 * n1);
+  const int fb = le * 6 * NF, fp0 = k * n1 + j, fp1 = k * n1 + i, fp2 = j * n1 + i;   // face points of the three lines
   double qq[5] = {0, 0, 0, 0, 0}, invJ = 0.0, rho_pt = 0.0;
+  double ja[3][3], g[12];
   if (active) {
 #pragma unroll
     for (int v = 0; v < 5; ++v) qq[v] = q[v * plane + gi];
     invJ = __ldg(met + 9 * plane + gi);
-    if (VISC)
 #pragma unroll
-      for (int k = 0; k < 4; ++k) sV[VISC ? le : 0][k][VISC ? pt : 0] = qq[k + 1];
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) ja[d][c] = __ldg(met + (3 * d + c) * plane + gi);
+    if (VISC && P > 0)
+#pragma unroll
+      for (int c = 0; c < 12; ++c) g[c] = __ldg(Gb + c * plane + gi);
   }
-  if (VISC) __syncthreads();
+  if (VISC) {
+    async_wait_all();
+    __syncthreads();
+  }
   if (active) {
-    double qa[5] = {qq[0] + ph.p_ref, qq[1], qq[2], qq[3], qq[4]};
-    rho_pt = qa[0] * s_rcp(qa[4]);
-    double ja[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) ja[i][c] = __ldg(met + (3 * i + c) * plane + gi);
-    double fv[12];
+    const double pabs = qq[0] + ph.p_ref;
+    rho_pt = pabs * s_rcp(qq[4]);
     if (VISC) {
-      const int i = pt % n1, j = (pt / n1) % n1, k = pt / (n1 * n1);
-      const int idx[3] = {i, j, k}, fpd[3] = {k * n1 + j, k * n1 + i, j * n1 + i};
-      double g[12];
+      double sj[3][3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) sj[d][c] = invJ * ja[d][c];
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
-        const double* V = sV[VISC ? le : 0][w];
-        double dr[3] = {0.0, 0.0, 0.0};
-        const double r0 = V[(k * n1 + j) * n1], r1 = V[k * n1 * n1 + i], r2 = V[j * n1 + i];
+        const double* Q = sQ[VISC ? w : 0] + (VISC ? fb : 0);
+        const double c0 = fma(sgL[i], Q[fp0], sgR[i] * Q[NF + fp0]);
+        const double c1 = fma(sgL[j], Q[2 * NF + fp1], sgR[j] * Q[3 * NF + fp1]);
+        const double c2 = fma(sgL[k], Q[4 * NF + fp2], sgR[k] * Q[5 * NF + fp2]);
 #pragma unroll
-        for (int m = 0; m < n1; ++m) {
-          dr[0] = fma(sD[i][m], V[(k * n1 + j) * n1 + m] - r0, dr[0]);
-          dr[1] = fma(sD[j][m], V[(k * n1 + m) * n1 + i] - r1, dr[1]);
-          dr[2] = fma(sD[k][m], V[(m * n1 + j) * n1 + i] - r2, dr[2]);
+        for (int c = 0; c < 3; ++c) {
+          const double t = fma(sj[0][c], c0, fma(sj[1][c], c1, sj[2][c] * c2));
+          g[c * 4 + w] = P > 0 ? g[c * 4 + w] + t : t;
         }
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          dr[d] = fma(sgL[idx[d]], __ldg(Qj + w * fplane + ((size_t)e * 6 + 2 * d) * NF + fpd[d]), dr[d]);
-          dr[d] = fma(sgR[idx[d]], __ldg(Qj + w * fplane + ((size_t)e * 6 + 2 * d + 1) * NF + fpd[d]), dr[d]);
-        }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) g[c * 4 + w] = invJ * (ja[0][c] * dr[0] + ja[1][c] * dr[1] + ja[2][c] * dr[2]);
       }
-      const double uvw[3] = {qq[1], qq[2], qq[3]};
-      viscous_flux3(uvw, g, ph, fv);
-    }
+      // Cartesian fluxes: momentum T = rho u u + pm I - tau (symmetric),
+      // energy rho u H - tau u - kT grad T
+      const double H = fma(ph.Cp, qq[4], 0.5 * fma(qq[1], qq[1], fma(qq[2], qq[2], qq[3] * qq[3])));
+      const double m2 = -2.0 * ph.mu, l23 = (ph.mu * (2.0 / 3.0)) * (g[0] + g[5] + g[10]);
+      double m[3], T[3][3], tt[3][3], en[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      double f[5];
-      flux3_n(qa, qq[0], ja[i], ph, f);
-      if (VISC)
+      for (int c = 0; c < 3; ++c) {
+        m[c] = rho_pt * qq[1 + c];
+        tt[c][c] = fma(m2, g[c * 4 + c], l23);
+        T[c][c] = fma(m[c], qq[1 + c], qq[0] + tt[c][c]);
+      }
 #pragma unroll
-        for (int r = 0; r < 4; ++r) f[r + 1] -= ja[i][0] * fv[r] + ja[i][1] * fv[4 + r] + ja[i][2] * fv[8 + r];
+      for (int c = 0; c < 3; ++c)
 #pragma unroll
-      for (int v = 0; v < 5; ++v) sF[le][i][v][pt] = f[v];
+        for (int d = c + 1; d < 3; ++d) {
+          tt[c][d] = tt[d][c] = -ph.mu * (g[c * 4 + d] + g[d * 4 + c]);
+          T[c][d] = T[d][c] = fma(m[c], qq[1 + d], tt[c][d]);
+        }
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        en[c] = fma(m[c], H, fma(-ph.kT, g[c * 4 + 3],
+                                 fma(qq[1], tt[c][0], fma(qq[2], tt[c][1], qq[3] * tt[c][2]))));
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        sF[le][d][0][pt] = fma(ja[d][0], m[0], fma(ja[d][1], m[1], ja[d][2] * m[2]));
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+          sF[le][d][1 + c][pt] = fma(ja[d][0], T[0][c], fma(ja[d][1], T[1][c], ja[d][2] * T[2][c]));
+        sF[le][d][4][pt] = fma(ja[d][0], en[0], fma(ja[d][1], en[1], ja[d][2] * en[2]));
+      }
+    } else {
+      const double H = fma(ph.Cp, qq[4], 0.5 * fma(qq[1], qq[1], fma(qq[2], qq[2], qq[3] * qq[3])));
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const double mn = rho_pt * fma(qq[1], ja[d][0], fma(qq[2], ja[d][1], qq[3] * ja[d][2]));
+        sF[le][d][0][pt] = mn;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) sF[le][d][1 + c][pt] = fma(mn, qq[1 + c], qq[0] * ja[d][c]);
+        sF[le][d][4][pt] = mn * H;
+      }
     }
   }
-  __syncthreads();
-  if (active) {
-    for (int it = pt; it < 30 * NF; it += N) {
-      const int f = it / (5 * NF), r = it - f * 5 * NF, v = r / NF, fp = r - v * NF;
-      const int a = fp % n1, b = fp / n1, d = f >> 1;
-      const bool plus = f & 1;
-      double loc = 0.0;
-#pragma unroll
-      for (int m = 0; m < n1; ++m) loc = fma(plus ? slp[m] : slm[m], sF[le][d][v][line_pt3<P>(f, a, b, m)], loc);
-      const double com = __ldg(Fcom + v * fplane + ((size_t)e * 6 + f) * NF + fp);
-      sJ[le][f][v][fp] = (plus ? com : -com) - loc;
-    }
-  }
+  if (!VISC) async_wait_all();
   __syncthreads();
   double ssq = 0.0;
   if (active) {
-    const int i = pt % n1, j = (pt / n1) % n1, k = pt / (n1 * n1);
+    const double ninvJ = -invJ;
     double qc[5];
     if (qn) {
       // q_c(q) - q_c(q_ref) with the energy through the pressure difference
@@ -322,13 +374,14 @@ __global__ void __launch_bounds__(64) volume3_kernel(int E, const double* q, con
         acc = fma(sD[j][m], sF[le][1][v][(k * n1 + m) * n1 + i], acc);
         acc = fma(sD[k][m], sF[le][2][v][(m * n1 + j) * n1 + i], acc);
       }
-      acc = fma(sgL[i], sJ[le][0][v][k * n1 + j], acc);
-      acc = fma(sgR[i], sJ[le][1][v][k * n1 + j], acc);
-      acc = fma(sgL[j], sJ[le][2][v][k * n1 + i], acc);
-      acc = fma(sgR[j], sJ[le][3][v][k * n1 + i], acc);
-      acc = fma(sgL[k], sJ[le][4][v][j * n1 + i], acc);
-      acc = fma(sgR[k], sJ[le][5][v][j * n1 + i], acc);
-      const double R = -acc * invJ;
+      const double* C = sC[v] + fb;   // outward: the -1 side's reference-direction flux is its negative
+      acc = fma(-sgL[i], C[fp0], acc);
+      acc = fma(sgR[i], C[NF + fp0], acc);
+      acc = fma(-sgL[j], C[2 * NF + fp1], acc);
+      acc = fma(sgR[j], C[3 * NF + fp1], acc);
+      acc = fma(-sgL[k], C[4 * NF + fp2], acc);
+      acc = fma(sgR[k], C[5 * NF + fp2], acc);
+      const double R = acc * ninvJ;
       const size_t o = v * plane + gi;
       if (mode == RES_PURE) {
         out[o] = R;
@@ -359,6 +412,7 @@ __global__ void __launch_bounds__(64) volume3_kernel(int E, const double* q, con
       // column's rows contiguously
       Acc acc[5] = {0, 0, 0, 0, 0};
       const W* Dm = Dinv + (size_t)e * n * n + pt;
+#pragma unroll 10
       for (int kk = 0; kk < n; ++kk) {
         const Acc rk = sr[APPLY ? le : 0][APPLY ? kk : 0];
 #pragma unroll
@@ -400,45 +454,66 @@ int residual_blocks_for3(int P, int E) {
 
 // Broken gradient of (u, v, w, T) at every solution point of hexahedra:
 // Gb[(c*4 + k) * E N + e N + pt], c = x, y, z, by the Lagrange derivative
-// along the three lines through the point (of the differences to each line's
-// first value: the derivative matrix annihilates constants, which keeps
-// T ~ 1/Ma^2 out of the rounding) and the chain rule with J a^i / |J|.
+// along the three lines through the point and the chain rule with J a^i / |J|.
+// The derivative is taken of the differences to the element's first value
+// (the derivative matrix annihilates constants, which keeps T ~ 1/Ma^2 out of
+// the rounding), formed once per value in shared memory.  Not run at P = 0,
+// where the gradient is zero.
 template <int P>
-__global__ void __launch_bounds__(128) grad3_kernel(int E, const double* __restrict__ q,
-                                                    const double* __restrict__ met, OpTab op,
-                                                    double* __restrict__ Gb) {
-  constexpr int n1 = P + 1, N = n1 * n1 * n1;
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= E * N) return;
-  const int e = tid / N, pt = tid - e * N, i = pt % n1, j = (pt / n1) % n1, k = pt / (n1 * n1);
-  const size_t plane = (size_t)E * N;
+struct GradEPB3 {
+  static constexpr int value = P == 1 ? 16 : P == 2 ? 7 : 2;   // 128, 189 (of 192), 128 points
+  static constexpr int threads = (value * (P + 1) * (P + 1) * (P + 1) + 31) / 32 * 32;
+};
+template <int P>
+__global__ void __launch_bounds__(GradEPB3<P>::threads) grad3_kernel(int E, const double* __restrict__ q,
+                                                                     const double* __restrict__ met, OpTab op,
+                                                                     double* __restrict__ Gb) {
+  constexpr int n1 = P + 1, N = n1 * n1 * n1, EPB = GradEPB3<P>::value;
+  __shared__ double sV[4][EPB * N];
+  __shared__ double sD[n1][n1];
+  const int e0 = blockIdx.x * EPB, np = min(EPB, E - e0) * N;
+  const size_t plane = (size_t)E * N, g0 = (size_t)e0 * N;
+  const int t = threadIdx.x, le = t / N, pt = t - le * N;
+  const int i = pt % n1, j = (pt / n1) % n1, k = pt / (n1 * n1);
+  const bool active = t < np;
+  if (t < n1 * n1) sD[t / n1][t % n1] = op.D[t / n1][t % n1];
   double ja[3][3];
+  if (active) {
+    const double iJ = __ldg(met + 9 * plane + g0 + t);
 #pragma unroll
-  for (int d = 0; d < 3; ++d)
+    for (int w = 0; w < 4; ++w) {
+      const double* V = q + (w + 1) * plane + g0;
+      sV[w][t] = __ldg(V + t) - __ldg(V + le * N);
+    }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) ja[d][c] = __ldg(met + (3 * d + c) * plane + tid);
-  const double iJ = __ldg(met + 9 * plane + tid);
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) ja[d][c] = iJ * __ldg(met + (3 * d + c) * plane + g0 + t);
+  }
+  __syncthreads();
+  if (!active) return;
 #pragma unroll
   for (int w = 0; w < 4; ++w) {
-    const double* V = q + (w + 1) * plane + (size_t)e * N;
-    const double r0 = __ldg(V + (k * n1 + j) * n1), r1 = __ldg(V + k * n1 * n1 + i), r2 = __ldg(V + j * n1 + i);
+    const double* V = sV[w] + le * N;
     double dr[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int m = 0; m < n1; ++m) {
-      dr[0] = fma(op.D[i][m], __ldg(V + (k * n1 + j) * n1 + m) - r0, dr[0]);
-      dr[1] = fma(op.D[j][m], __ldg(V + (k * n1 + m) * n1 + i) - r1, dr[1]);
-      dr[2] = fma(op.D[k][m], __ldg(V + (m * n1 + j) * n1 + i) - r2, dr[2]);
+      dr[0] = fma(sD[i][m], V[(k * n1 + j) * n1 + m], dr[0]);
+      dr[1] = fma(sD[j][m], V[(k * n1 + m) * n1 + i], dr[1]);
+      dr[2] = fma(sD[k][m], V[(m * n1 + j) * n1 + i], dr[2]);
     }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) Gb[(c * 4 + w) * plane + tid] = iJ * (ja[0][c] * dr[0] + ja[1][c] * dr[1] + ja[2][c] * dr[2]);
+    for (int c = 0; c < 3; ++c)
+      Gb[(c * 4 + w) * plane + g0 + t] = fma(ja[0][c], dr[0], fma(ja[1][c], dr[1], ja[2][c] * dr[2]));
   }
 }
 
 void launch_grad3(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s) {
-  const int total = c.E * L.N, threads = 128, blocks = (total + threads - 1) / threads;
-#define PMG_G3(PP) grad3_kernel<PP><<<blocks, threads, 0, s>>>(c.E, q, L.met, L.op, L.Gb)
+#define PMG_G3(PP)                                                                                            \
+  grad3_kernel<PP><<<(c.E + GradEPB3<PP>::value - 1) / GradEPB3<PP>::value, GradEPB3<PP>::threads, 0, s>>>( \
+      c.E, q, L.met, L.op, L.Gb)
   switch (L.P) {
-    case 0: PMG_G3(0); break;
+    case 0: break;   // zero
     case 1: PMG_G3(1); break;
     case 2: PMG_G3(2); break;
     default: PMG_G3(3); break;
@@ -474,11 +549,11 @@ void launch_volume3(const Ctx& c, const LevelDev& L, const double* q, double* ou
 #define PMG_V3(PP)                                                                                               \
   if (visc)                                                                                                      \
     volume3_kernel<PP, double, false, true><<<blocks, threads3<PP>(), 0, s>>>(                                  \
-        c.E, q, L.met, L.Fcom, L.Qj, L.op, c.ph, out, (int)mode, inv_odt, src, S, Sout, Pd, qn, partial, nullptr, \
+        c.E, q, L.met, L.Fcom, L.Qj, L.Gb, L.op, c.ph, out, (int)mode, inv_odt, src, S, Sout, Pd, qn, partial, nullptr, \
         nullptr, nullptr, nullptr);                                                                              \
   else                                                                                                           \
     volume3_kernel<PP, double, false, false><<<blocks, threads3<PP>(), 0, s>>>(                                 \
-        c.E, q, L.met, L.Fcom, nullptr, L.op, c.ph, out, (int)mode, inv_odt, src, S, Sout, Pd, qn, partial,      \
+        c.E, q, L.met, L.Fcom, nullptr, nullptr, L.op, c.ph, out, (int)mode, inv_odt, src, S, Sout, Pd, qn, partial,      \
         nullptr, nullptr, nullptr, nullptr)
   switch (L.P) {
     case 0: PMG_V3(0); break;
@@ -498,11 +573,11 @@ static void volume_apply3_dispatch(const Ctx& c, const LevelDev& L, double* q, d
 #define PMG_VA3(PP)                                                                                             \
   if (visc)                                                                                                     \
     volume3_kernel<PP, W, true, true><<<blocks, threads3<PP>(), 0, s>>>(                                       \
-        c.E, q, L.met, L.Fcom, L.Qj, L.op, c.ph, nullptr, (int)RES_SYSTEM, inv_odt, src, S, nullptr, nullptr, qn, \
+        c.E, q, L.met, L.Fcom, L.Qj, L.Gb, L.op, c.ph, nullptr, (int)RES_SYSTEM, inv_odt, src, S, nullptr, nullptr, qn, \
         nullptr, q, Dinv, L.rs, L.cs);                                                                          \
   else                                                                                                          \
     volume3_kernel<PP, W, true, false><<<blocks, threads3<PP>(), 0, s>>>(                                      \
-        c.E, q, L.met, L.Fcom, nullptr, L.op, c.ph, nullptr, (int)RES_SYSTEM, inv_odt, src, S, nullptr, nullptr, \
+        c.E, q, L.met, L.Fcom, nullptr, nullptr, L.op, c.ph, nullptr, (int)RES_SYSTEM, inv_odt, src, S, nullptr, nullptr, \
         qn, nullptr, q, Dinv, L.rs, L.cs)
   switch (L.P) {
     case 0: PMG_VA3(0); break;

@@ -8,10 +8,10 @@
 //
 //  1. own state and contravariant fluxes to shared memory;
 //  2. the element's own 4 (P+1) face points: own and neighbour traces (the
-//     neighbour from the input state), preconditioned Roe flux, jump against
-//     the extrapolated flux polynomial.  Each face is evaluated by both of
+//     neighbour from the input state), preconditioned Roe flux.  Each face is evaluated by both of
 //     its elements: twice the face arithmetic, but no grid-wide dependency;
-//  3. divergence + DG correction, level-system epilogue (F - S, stage term
+//  3. divergence of each line, Dt F + gL F_com(-1) + gR F_com(+1) (at P = 0
+//     Dt is zero: the face fluxes alone), level-system epilogue (F - S, stage term
 //     relative to q^b or q^n);
 //  4. x = cs .* (D^-1 (rs .* F)) with the element's factored block, written to
 //     a second state buffer (Jacobi: every element reads the old state).
@@ -94,9 +94,9 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_kernel(
       for (int v = 0; v < 4; ++v) qo[v] = __ldg(qref + v * plane + (size_t)e_0 * N + t0);
     }
   }
-  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = op.D[threadIdx.x / n1][threadIdx.x % n1];
+  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = op.Dt[threadIdx.x / n1][threadIdx.x % n1];
   if (threadIdx.x < n1) {
-    sgL[threadIdx.x] = op.gL[threadIdx.x];
+    sgL[threadIdx.x] = -op.gL[threadIdx.x];   // the fluxes are outward
     sgR[threadIdx.x] = op.gR[threadIdx.x];
     slm[threadIdx.x] = op.lm[threadIdx.x];
     slp[threadIdx.x] = op.lp[threadIdx.x];
@@ -113,12 +113,14 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_kernel(
       double qa[4] = {qq[0] + ph.p_ref, qq[1], qq[2], qq[3]};
       double a = __ldg(met + gi), b = __ldg(met + plane + gi);
       double c = __ldg(met + 2 * plane + gi), d = __ldg(met + 3 * plane + gi);
-      double f[4], g[4];
-      flux_xy(qa, qq[0], ph, f, g);
+      if (P > 0) {   // at P = 0 the line operator Dt is zero
+        double f[4], g[4];
+        flux_xy(qa, qq[0], ph, f, g);
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        sFt[le][v][t] = fma(a, f[v], b * g[v]);
-        sGt[le][v][t] = fma(c, f[v], d * g[v]);
+        for (int v = 0; v < 4; ++v) {
+          sFt[le][v][t] = fma(a, f[v], b * g[v]);
+          sGt[le][v][t] = fma(c, f[v], d * g[v]);
+        }
       }
     }
   }
@@ -129,7 +131,7 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_kernel(
     const int e = blockIdx.x * EPB + le;
     if (le < EPB && e < E) {
       const int f = t / n1, k = t - f * n1;
-      const bool plus = (f == 1 || f == 2), eta = (f == 0 || f == 2), xi = !eta;
+      const bool plus = (f == 1 || f == 2), eta = (f == 0 || f == 2);
       const double ref[4] = {sq[le][0][0], 0.0, 0.0, sq[le][3][0]};
       double sm[4], sp[4];
 #pragma unroll
@@ -158,13 +160,7 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_kernel(
       double out[4];
       face_roe<DWF>(qm, qp, dq, pgm, pgp, gx, gy, gS, ph, phw, out);
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        double loc = 0.0;
-#pragma unroll
-        for (int m = 0; m < n1; ++m)
-          loc = fma(plus ? slp[m] : slm[m], xi ? sFt[le][v][k * n1 + m] : sGt[le][v][m * n1 + k], loc);
-        sJ[le][f][v][k] = (plus ? out[v] : -out[v]) - loc;
-      }
+      for (int v = 0; v < 4; ++v) sJ[le][f][v][k] = out[v];   // outward
     }
   }
   __syncthreads();
@@ -194,11 +190,12 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_kernel(
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         double acc = 0.0;
+        if (P > 0)
 #pragma unroll
-        for (int m = 0; m < n1; ++m) {
-          acc = fma(sD[i][m], sFt[le][v][j * n1 + m], acc);
-          acc = fma(sD[j][m], sGt[le][v][m * n1 + i], acc);
-        }
+          for (int m = 0; m < n1; ++m) {
+            acc = fma(sD[i][m], sFt[le][v][j * n1 + m], acc);
+            acc = fma(sD[j][m], sGt[le][v][m * n1 + i], acc);
+          }
         acc = fma(sgL[i], sJ[le][3][v][j], acc);
         acc = fma(sgR[i], sJ[le][1][v][j], acc);
         acc = fma(sgL[j], sJ[le][0][v][i], acc);
@@ -241,8 +238,7 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_kernel(
 }
 
 // The same sweep in double-word arithmetic (gauge storage, the sweeps of
-// PMG_FLUX_DW_SMOOTH): contravariant fluxes, face fluxes, face jumps, the
-// divergence and the level-system epilogue run on the FP32 pipes (dword.cuh;
+// PMG_FLUX_DW_SMOOTH): contravariant fluxes, face fluxes, the divergence and the level-system epilogue run on the FP32 pipes (dword.cuh;
 // see k_volume_dw.cu), while the traces and jumps the face flux takes are
 // still formed in binary64 relative to the element's first point.
 template <int P, class W>
@@ -264,7 +260,7 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
   using Acc = typename Blk<W>::acc;
   __shared__ Acc sr[EPB][n];
   __shared__ double slm[n1], slp[n1];
-  __shared__ dw sD[n1][n1], sgL[n1], sgR[n1], swm[n1], swp[n1];
+  __shared__ dw sD[n1][n1], sgL[n1], sgR[n1];
   const size_t plane = (size_t)E * N;
   if (threadIdx.x == 0) {
     const int e0 = blockIdx.x * EPB, ne = min(EPB, E - e0);
@@ -311,12 +307,10 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
 #pragma unroll
     for (int c = 0; c < 5; ++c) mt[c] = __ldg(met + c * plane + gi);
   }
-  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = opw.D[threadIdx.x / n1][threadIdx.x % n1];
+  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = opw.Dt[threadIdx.x / n1][threadIdx.x % n1];
   if (threadIdx.x < n1) {
-    sgL[threadIdx.x] = opw.gL[threadIdx.x];
+    sgL[threadIdx.x] = -opw.gL[threadIdx.x];   // the fluxes are outward
     sgR[threadIdx.x] = opw.gR[threadIdx.x];
-    swm[threadIdx.x] = opw.lm[threadIdx.x];
-    swp[threadIdx.x] = opw.lp[threadIdx.x];
     slm[threadIdx.x] = op.lm[threadIdx.x];
     slp[threadIdx.x] = op.lp[threadIdx.x];
   }
@@ -330,29 +324,30 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
       Q[v] = dw_from_double(qq[v]);   // gauge p, u, v, T
     }
     rho = (Q[0] + k.p_ref) * rcp(Q[3]);
-    const dw a = dw_from_double(mt[0]), b = dw_from_double(mt[1]);
-    const dw c = dw_from_double(mt[2]), d = dw_from_double(mt[3]);
-    const dw H = k.Cp * Q[3] + half(Q[1] * Q[1] + Q[2] * Q[2]);
-    const dw mx = rho * Q[1], my = rho * Q[2];
-    const dw fx[4] = {mx, mx * Q[1] + Q[0], mx * Q[2], mx * H};
-    const dw gy4[4] = {my, my * Q[1], my * Q[2] + Q[0], my * H};
+    if (P > 0) {   // at P = 0 the line operator Dt is zero
+      const dw a = dw_from_double(mt[0]), b = dw_from_double(mt[1]);
+      const dw c = dw_from_double(mt[2]), d = dw_from_double(mt[3]);
+      const dw H = k.Cp * Q[3] + half(Q[1] * Q[1] + Q[2] * Q[2]);
+      const dw mx = rho * Q[1], my = rho * Q[2];
+      const dw fx[4] = {mx, mx * Q[1] + Q[0], mx * Q[2], mx * H};
+      const dw gy4[4] = {my, my * Q[1], my * Q[2] + Q[0], my * H};
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      dw_acc x, y;
-      x.add_prod(a, fx[v]);
-      x.add_prod(b, gy4[v]);
-      y.add_prod(c, fx[v]);
-      y.add_prod(d, gy4[v]);
-      sFt[le][v][t] = x.value();
-      sGt[le][v][t] = y.value();
+      for (int v = 0; v < 4; ++v) {
+        dw_acc x, y;
+        x.add_prod(a, fx[v]);
+        x.add_prod(b, gy4[v]);
+        y.add_prod(c, fx[v]);
+        y.add_prod(d, gy4[v]);
+        sFt[le][v][t] = x.value();
+        sGt[le][v][t] = y.value();
+      }
     }
   }
   __syncthreads();
   // phase 2: face point (f, kf): binary64 traces relative to the element's
-  // first point, the double-word face flux, the jump against the extrapolated
-  // flux polynomial
+  // first point, the double-word face flux
   if (act) {
-    const bool plus = (f == 1 || f == 2), eta = (f == 0 || f == 2), xi = !eta;
+    const bool plus = (f == 1 || f == 2), eta = (f == 0 || f == 2);
     const double ref[4] = {sq[le][0][0], 0.0, 0.0, sq[le][3][0]};
     double sm[4], sp[4];
     const bool pn = (fn == 1 || fn == 2);
@@ -380,13 +375,7 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
     dw out[4];
     face_roe_dw(qm, qp, dq, pgm, pgp, gx, gy, gS, k, out);
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      dw_acc loc;
-#pragma unroll
-      for (int m = 0; m < n1; ++m)
-        loc.add_prod(plus ? swp[m] : swm[m], xi ? sFt[le][v][kf * n1 + m] : sGt[le][v][m * n1 + kf]);
-      sJ[le][f][v][kf] = (plus ? out[v] : -out[v]) - loc.value();
-    }
+    for (int v = 0; v < 4; ++v) sJ[le][f][v][kf] = out[v];   // outward
   }
   __syncthreads();
   const bool ok = mbar_wait0(&mbar, k.wait_ns);
@@ -416,11 +405,12 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
       dw_acc acc;
+      if (P > 0)
 #pragma unroll
-      for (int m = 0; m < n1; ++m) {
-        acc.add_prod(sD[i][m], sFt[le][v][j * n1 + m]);
-        acc.add_prod(sD[j][m], sGt[le][v][m * n1 + i]);
-      }
+        for (int m = 0; m < n1; ++m) {
+          acc.add_prod(sD[i][m], sFt[le][v][j * n1 + m]);
+          acc.add_prod(sD[j][m], sGt[le][v][m * n1 + i]);
+        }
       acc.add_prod(sgL[i], sJ[le][3][v][j]);
       acc.add_prod(sgR[i], sJ[le][1][v][j]);
       acc.add_prod(sgL[j], sJ[le][0][v][i]);

@@ -8,9 +8,9 @@
 //    On a boundary face the outer state is the ghost state of the boundary
 //    type (physics.cuh ghost_state), formed here relative to the reference.
 //  * volume: one thread per solution point, several elements per CTA.
-//    Contravariant fluxes go to shared memory; the Lagrange derivative, the
-//    face jumps (common minus extrapolated flux polynomial) and the DG
-//    correction are applied there, followed by the epilogue of the requested
+//    Contravariant fluxes go to shared memory; a line's divergence is
+//    Dt F + gL F_com(-1) + gR F_com(+1), the derivative with the extrapolated
+//    part of the DG correction folded in (OpTab::Dt), followed by the epilogue of the requested
 //    mode (pure R, level system residual, FAS forcing) and an optional
 //    deterministic per-CTA sum of squares for the residual norm.
 //
@@ -18,6 +18,13 @@
 // TFLOP/s).  The face kernel's double-word variant (face_roe<true>, the
 // element-Jacobi sweeps) runs the Roe flux on the FP32 pipes; the sweeps'
 // residual-and-update in double-word is k_volume_dw.cu.
+//
+// An FP64 warp instruction takes 64 cycles of its sub-partition whatever lanes
+// are active, so the kernels are timed by their count: no face jumps are
+// formed, the viscous launches add only the face corrections to the broken
+// gradient already written.  Full-size cylinder residual (16384 quadrilaterals,
+// P = 4, viscous; one GB300): gradient 62 -> 38 us, face flux 118 -> 106 us,
+// residual 215 -> 136 us.
 //
 // Viscous terms (mu > 0, Section 2.1 fluxes, Section 2.3 common viscous flux):
 // a gradient launch (k_viscous.cu) first forms the broken gradients of
@@ -56,7 +63,8 @@ __device__ __forceinline__ void line_trace(const double* __restrict__ q, size_t 
   }
 }
 
-// Trace of the six broken-gradient planes of element e at face point (f, k).
+// Adds the trace of the six broken-gradient planes of element e at face point
+// (f, k) to out, with the trace weights lm, lp given.
 template <int P>
 __device__ __forceinline__ void grad_trace(const double* __restrict__ Gb, size_t plane, int e, int f, int k,
                                            const double* lm, const double* lp, double out[6]) {
@@ -67,14 +75,14 @@ __device__ __forceinline__ void grad_trace(const double* __restrict__ Gb, size_t
   const int stride = eta ? n1 : 1;
 #pragma unroll
   for (int v = 0; v < 6; ++v) {
-    double s = 0.0;
 #pragma unroll
-    for (int m = 0; m < n1; ++m) s = fma(plus ? lp[m] : lm[m], __ldg(base + v * plane + m * stride), s);
-    out[v] = s;
+    for (int m = 0; m < n1; ++m) out[v] = fma(plus ? lp[m] : lm[m], __ldg(base + v * plane + m * stride), out[v]);
   }
 }
 
-template <int P, bool VISC, bool DWF>
+// OUTDW: the fluxes are left as double-words for volume_apply_dw_kernel
+// (sweeps with gauge storage and mu = 0).
+template <int P, bool VISC, bool DWF, bool OUTDW>
 __global__ void __launch_bounds__(256) face_flux_kernel(const int* __restrict__ faces, int n_faces, int E,
                                                         const double* __restrict__ q,
                                                         const double* __restrict__ face,
@@ -129,29 +137,37 @@ __global__ void __launch_bounds__(256) face_flux_kernel(const int* __restrict__ 
   const double pgm = qm[0], pgp = qp[0];   // gauge pressures for the momentum fluxes
   qm[0] += ph.p_ref;   // absolute pressure for the averaged state and rho
   qp[0] += ph.p_ref;
-  double out[4];
-  face_roe<DWF>(qm, qp, dq, pgm, pgp, nx, ny, dS, ph, phw, out);
   const size_t fplane = (size_t)E * 4 * n1;
   const size_t iL = ((size_t)eL * 4 + fL) * n1 + k;
   const size_t iR = bnd ? iL : ((size_t)eR * 4 + fR) * n1 + kR;
+  if (OUTDW) {
+    dw o[4];
+    face_roe_dw(qm, qp, dq, pgm, pgp, nx, ny, dS, phw, o);
+    dw* Fw = reinterpret_cast<dw*>(Fcom);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      Fw[v * fplane + iL] = o[v];
+      if (!bnd) Fw[v * fplane + iR] = -o[v];
+    }
+    return;
+  }
+  double out[4];
+  face_roe<DWF>(qm, qp, dq, pgm, pgp, nx, ny, dS, ph, phw, out);
   if (VISC) {
     // common gradient: mean of the two broken-gradient traces plus the BR2
     // liftings r^- + r^+ = pen (q_com - q^-) (1/|J|^- + 1/|J|^+) n dS, with
     // q_com - q^- = dq / 2.  A boundary face mirrors the element (its
     // gradient trace and |J|): the one-sided BR2 gradient.
-    double gm[6], gp[6], gc[6];
-    grad_trace<P>(Gb, plane, eL, fL, k, lm, lp, gm);
-    if (!bnd) {
-      grad_trace<P>(Gb, plane, eR, fR, kR, lm, lp, gp);
-    } else {
-#pragma unroll
-      for (int c = 0; c < 6; ++c) gp[c] = gm[c];
-    }
     const double wl = 0.25 * op.pen * (__ldg(fJinv + iL) + __ldg(fJinv + iR)) * dS;
+    double gc[6];
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
-      gc[v] = fma(wl * nx, dq[v + 1], 0.5 * (gm[v] + gp[v]));
-      gc[3 + v] = fma(wl * ny, dq[v + 1], 0.5 * (gm[3 + v] + gp[3 + v]));
+      gc[v] = (wl * nx) * dq[v + 1];
+      gc[3 + v] = (wl * ny) * dq[v + 1];
+    }
+    if (P > 0) {   // at P = 0 the broken gradient is zero
+      grad_trace<P>(Gb, plane, eL, fL, k, op.hlm, op.hlp, gc);
+      grad_trace<P>(Gb, plane, bnd ? eL : eR, bnd ? fL : fR, bnd ? k : kR, op.hlm, op.hlp, gc);
     }
     double fv[4], gv[4];
     viscous_flux(0.5 * (qm[1] + qp[1]), 0.5 * (qm[2] + qp[2]), gc, ph, fv, gv);
@@ -190,7 +206,7 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
                                                      double* __restrict__ partial, double* qw,
                                                      const W* __restrict__ Dinv, const double* __restrict__ rs,
                                                      const double* __restrict__ cs,
-                                                     const double* __restrict__ Qj,
+                                                     const double* __restrict__ Qj, const double* __restrict__ Gb,
                                                      double* __restrict__ werr) {
   constexpr int n1 = P + 1, N = n1 * n1, EPB = ElemsPerBlock<P>::value, n = 4 * N;
   using PF = VolPrefetch<P, W>;
@@ -198,11 +214,9 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
   __shared__ __align__(8) unsigned long long mbar[2];   // 0: face fluxes, 1: blocks and scales
   using Acc = typename Blk<W>::acc;
   __shared__ Acc sr[APPLY ? EPB : 1][APPLY ? n : 1];
-  __shared__ double sV[VISC ? EPB : 1][3][VISC ? N : 1];   // (u, v, T) for the gradients
   __shared__ double sFt[EPB][4][N];
   __shared__ double sGt[EPB][4][N];
-  __shared__ double sJ[EPB][4][4][n1];   // [face][var][k]
-  __shared__ double sD[n1][n1], sgL[n1], sgR[n1], slm[n1], slp[n1];
+  __shared__ double sD[n1][n1], sgL[n1], sgR[n1];   // Dt, gL, gR
   __shared__ double sred[256 / 32];
 
   const int le = threadIdx.x / N, pt = threadIdx.x - le * N;
@@ -241,23 +255,15 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
       if (S) Sv[v] = __ldg(S + v * plane + g0);
     }
   }
-  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = op.D[threadIdx.x / n1][threadIdx.x % n1];
+  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = op.Dt[threadIdx.x / n1][threadIdx.x % n1];
   if (threadIdx.x < n1) {
     sgL[threadIdx.x] = op.gL[threadIdx.x];
     sgR[threadIdx.x] = op.gR[threadIdx.x];
-    slm[threadIdx.x] = op.lm[threadIdx.x];
-    slp[threadIdx.x] = op.lp[threadIdx.x];
   }
 
   double qq[4] = {0, 0, 0, 0}, invJ = 0.0, rho_pt = 0.0;
   size_t gi = (size_t)e * N + pt;
-  if (VISC) {
-    if (active) {
-#pragma unroll
-      for (int v = 1; v < 4; ++v) sV[VISC ? le : 0][v - 1][VISC ? pt : 0] = q[v * plane + gi];
-    }
-    __syncthreads();
-  }
+  if (VISC) __syncthreads();   // sgL, sgR
   if (active) {
 #pragma unroll
     for (int v = 0; v < 4; ++v) qq[v] = q[v * plane + gi];
@@ -269,26 +275,20 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
     double f[4], g[4];
     flux_xy_rho(qa, qq[0], rho_pt, ph, f, g);
     if (VISC) {
-      // corrected gradient: reference derivatives plus the DG correction of
-      // the jumps q_com - q_own at the four faces' points on this point's lines
+      // corrected gradient: the broken gradient of the gradient launch plus
+      // the DG correction of the jumps q_com - q_own at the four faces'
+      // points on this point's lines
       const int i = pt % n1, j = pt / n1;
       const double* Qe = Qj + (size_t)e * 4 * n1;
+      const double ia = invJ * a, ib = invJ * b, ic = invJ * c, id = invJ * d;
       double gr[6], fv[4], gv[4];
 #pragma unroll
       for (int v = 0; v < 3; ++v) {
-        double ax = 0.0, ae = 0.0;
-#pragma unroll
-        for (int m = 0; m < n1; ++m) {   // differences to the line's first value
-          ax = fma(sD[i][m], sV[VISC ? le : 0][v][VISC ? j * n1 + m : 0] - sV[VISC ? le : 0][v][VISC ? j * n1 : 0], ax);
-          ae = fma(sD[j][m], sV[VISC ? le : 0][v][VISC ? m * n1 + i : 0] - sV[VISC ? le : 0][v][VISC ? i : 0], ae);
-        }
         const double* Qv = Qe + v * fplane;
-        ax = fma(sgL[i], __ldg(Qv + 3 * n1 + j), ax);
-        ax = fma(sgR[i], __ldg(Qv + 1 * n1 + j), ax);
-        ae = fma(sgL[j], __ldg(Qv + 0 * n1 + i), ae);
-        ae = fma(sgR[j], __ldg(Qv + 2 * n1 + i), ae);
-        gr[v] = invJ * fma(a, ax, c * ae);
-        gr[3 + v] = invJ * fma(b, ax, d * ae);
+        const double cx = fma(sgL[i], __ldg(Qv + 3 * n1 + j), sgR[i] * __ldg(Qv + 1 * n1 + j));
+        const double ce = fma(sgL[j], __ldg(Qv + 0 * n1 + i), sgR[j] * __ldg(Qv + 2 * n1 + i));
+        gr[v] = fma(ia, cx, P > 0 ? fma(ic, ce, __ldg(Gb + v * plane + gi)) : ic * ce);
+        gr[3 + v] = fma(ib, cx, P > 0 ? fma(id, ce, __ldg(Gb + (3 + v) * plane + gi)) : id * ce);
       }
       viscous_flux(qq[1], qq[2], gr, ph, fv, gv);
 #pragma unroll
@@ -303,29 +303,12 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
   __syncthreads();
   const bool okF = APPLY ? mbar_wait0(&mbar[0], ph.wait_ns) : true;
   if (!okF) *werr = 1.0;
-  if (active) {
-    // face jumps: common (reference-direction) minus extrapolated flux polynomial
-    for (int it = pt; it < 16 * n1; it += N) {
-      int f = it / (4 * n1), r = it - f * 4 * n1, v = r / n1, k = r - v * n1;
-      const bool xi = (f == 1 || f == 3);
-      const bool plus = (f == 1 || f == 2);
-      double loc = 0.0;
-#pragma unroll
-      for (int m = 0; m < n1; ++m) {
-        double fv = xi ? sFt[le][v][k * n1 + m] : sGt[le][v][m * n1 + k];
-        loc = fma(plus ? slp[m] : slm[m], fv, loc);
-      }
-      double com = (APPLY && okF) ? sFc[((v * EPB + le) * 4 + f) * n1 + k]
-                                  : __ldg(Fcom + v * fplane + ((size_t)e * 4 + f) * n1 + k);
-      sJ[le][f][v][k] = (plus ? com : -com) - loc;
-    }
-  }
-  __syncthreads();
   const bool okS = APPLY ? mbar_wait0(&mbar[1], ph.wait_ns) : true;
   if (!okS) *werr = 1.0;
   double ssq = 0.0;
   if (active) {
     const int i = pt % n1, j = pt / n1;
+    const double ninvJ = -invJ;
     double qc[4];
     if (qn) {
       // q_c(q) - q_c(q_ref) with the energy difference taken through
@@ -356,11 +339,18 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
         acc = fma(sD[i][m], sFt[le][v][j * n1 + m], acc);
         acc = fma(sD[j][m], sGt[le][v][m * n1 + i], acc);
       }
-      acc = fma(sgL[i], sJ[le][3][v][j], acc);
-      acc = fma(sgR[i], sJ[le][1][v][j], acc);
-      acc = fma(sgL[j], sJ[le][0][v][i], acc);
-      acc = fma(sgR[j], sJ[le][2][v][i], acc);
-      double R = -acc * invJ;
+      double com[4];   // outward: the -1 sides' reference-direction fluxes are their negatives
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const int kk = (f == 1 || f == 3) ? j : i;
+        com[f] = (APPLY && okF) ? sFc[((v * EPB + le) * 4 + f) * n1 + kk]
+                                : __ldg(Fcom + v * fplane + ((size_t)e * 4 + f) * n1 + kk);
+      }
+      acc = fma(-sgL[i], com[3], acc);
+      acc = fma(sgR[i], com[1], acc);
+      acc = fma(-sgL[j], com[0], acc);
+      acc = fma(sgR[j], com[2], acc);
+      double R = acc * ninvJ;
       size_t o = v * plane + gi;
       if (mode == RES_PURE) {
         out[o] = R;
@@ -490,18 +480,20 @@ void launch_face_flux(const Ctx& c, const LevelDev& L, const double* q, cudaStre
   int threads = 32, blocks = (total + threads - 1) / threads;
   const bool visc = c.ph.mu > 0.0, dwf = sweep ? flux_dw_sweep(c) : flux_dw(c, L);
   if (visc) launch_grad(c, L, q, s);
-#define PMG_FACE_V(PP, V, D)                                                                                 \
-  face_flux_kernel<PP, V, D><<<blocks, threads, 0, s>>>(c.d_faces, c.n_faces, c.E, q, L.face, L.Fcom, L.op, \
+  const bool outdw = sweep && volume_dw_applies(c);
+#define PMG_FACE_V(PP, V, D, O)                                                                              \
+  face_flux_kernel<PP, V, D, O><<<blocks, threads, 0, s>>>(c.d_faces, c.n_faces, c.E, q, L.face, L.Fcom, L.op, \
                                                         c.ph, c.phw, V ? L.Gb : nullptr,                    \
                                                         V ? L.fJinv : nullptr, V ? L.Qj : nullptr)
 #define PMG_FACE(PP)                                   \
   do {                                                 \
     if (visc) {                                        \
-      if (dwf) PMG_FACE_V(PP, true, true);             \
-      else PMG_FACE_V(PP, true, false);                \
+      if (dwf) PMG_FACE_V(PP, true, true, false);      \
+      else PMG_FACE_V(PP, true, false, false);         \
     } else {                                           \
-      if (dwf) PMG_FACE_V(PP, false, true);            \
-      else PMG_FACE_V(PP, false, false);               \
+      if (outdw) PMG_FACE_V(PP, false, true, true);    \
+      else if (dwf) PMG_FACE_V(PP, false, true, false); \
+      else PMG_FACE_V(PP, false, false, false);        \
     }                                                  \
   } while (0)
   switch (L.P) {
@@ -528,11 +520,11 @@ void launch_volume(const Ctx& c, const LevelDev& L, int level, const double* q, 
     if (c.ph.mu > 0.0)                                                                                       \
       volume_kernel<PP, double, false, true><<<blocks, threads, 0, s>>>(                                     \
           c.E, q, L.met, L.Fcom, L.op, c.ph, out, (int)mode, inv_odt, src, S, Sout, Pd, qn, partial, nullptr, \
-          nullptr, nullptr, nullptr, L.Qj, nullptr);                                                         \
+          nullptr, nullptr, nullptr, L.Qj, L.Gb, nullptr);                                                         \
     else                                                                                                     \
       volume_kernel<PP, double, false, false><<<blocks, threads, 0, s>>>(                                    \
           c.E, q, L.met, L.Fcom, L.op, c.ph, out, (int)mode, inv_odt, src, S, Sout, Pd, qn, partial, nullptr, \
-          nullptr, nullptr, nullptr, nullptr, nullptr);                                                      \
+          nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);                                             \
   } while (0)
   switch (L.P) {
     case 0: PMG_VOL(0); break;
@@ -559,12 +551,12 @@ static void volume_apply_dispatch(const Ctx& c, const LevelDev& L, double* q, do
       volume_kernel<PP, W, true, true><<<blocks, threads, sm, s>>>(c.E, q, L.met, L.Fcom, L.op, c.ph, nullptr,  \
                                                                    (int)RES_SYSTEM, inv_odt, src, S, nullptr,   \
                                                                    nullptr, qn, nullptr, q, Dinv, L.rs, L.cs,   \
-                                                                   L.Qj, werr);                                 \
+                                                                   L.Qj, L.Gb, werr);                           \
     else                                                                                                       \
       volume_kernel<PP, W, true, false><<<blocks, threads, sm, s>>>(c.E, q, L.met, L.Fcom, L.op, c.ph, nullptr, \
                                                                     (int)RES_SYSTEM, inv_odt, src, S, nullptr,  \
                                                                     nullptr, qn, nullptr, q, Dinv, L.rs, L.cs,  \
-                                                                    nullptr, werr);                             \
+                                                                    nullptr, nullptr, werr);                    \
   } while (0)
   switch (L.P) {
     case 0: PMG_VA(0); break;

@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
   Acc* sr = reinterpret_cast<Acc*>(sDinv + (size_t)M * n * n); // [M][n]
   int* slnb = reinterpret_cast<int*>(sr + (size_t)M * n);      // [M][4]
   int* sfn = slnb + (size_t)M * 4;                   // [M][4]: neighbour face | reversed << 3
-  __shared__ dw sD[n1][n1], sgL[n1], sgR[n1], swm[n1], swp[n1];
+  __shared__ dw sD[n1][n1], sgL[n1], sgR[n1];
   __shared__ double slm[n1], slp[n1];
   const size_t plane = (size_t)E * N;
 
@@ -108,12 +108,10 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
       for (int c = 0; c < 5; ++c) smt[((size_t)slot * 5 + c) * N + tf] = __ldg(met + c * plane + gi);
     }
   }
-  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = opw.D[threadIdx.x / n1][threadIdx.x % n1];
+  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = opw.Dt[threadIdx.x / n1][threadIdx.x % n1];
   if (threadIdx.x < n1) {
-    sgL[threadIdx.x] = opw.gL[threadIdx.x];
+    sgL[threadIdx.x] = -opw.gL[threadIdx.x];   // the fluxes are outward
     sgR[threadIdx.x] = opw.gR[threadIdx.x];
-    swm[threadIdx.x] = opw.lm[threadIdx.x];
-    swp[threadIdx.x] = opw.lp[threadIdx.x];
     slm[threadIdx.x] = op.lm[threadIdx.x];
     slp[threadIdx.x] = op.lp[threadIdx.x];
   }
@@ -151,7 +149,7 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
     __syncthreads();
     // phase 2: face point (f, kf), the neighbour from the tile
     if (act) {
-      const bool plus = (f == 1 || f == 2), eta = (f == 0 || f == 2), xi = !eta;
+      const bool plus = (f == 1 || f == 2), eta = (f == 0 || f == 2);
       const double* sqe = sqA + (size_t)slot * 4 * N;
       const double ref[4] = {sqe[0], 0.0, 0.0, sqe[3 * N]};
       const int ln = slnb[slot * 4 + f], fnr = sfn[slot * 4 + f];
@@ -184,14 +182,7 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
       dw out[4];
       face_roe_dw(qm, qp, dq, pgm, pgp, g[0], g[1], g[2], k, out);
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        dw_acc loc;
-#pragma unroll
-        for (int m = 0; m < n1; ++m)
-          loc.add_prod(plus ? swp[m] : swm[m], xi ? sFt[((size_t)slot * 4 + v) * N + kf * n1 + m]
-                                                  : sGt[((size_t)slot * 4 + v) * N + m * n1 + kf]);
-        sJ[(((size_t)slot * 4 + f) * 4 + v) * n1 + kf] = (plus ? out[v] : -out[v]) - loc.value();
-      }
+      for (int v = 0; v < 4; ++v) sJ[(((size_t)slot * 4 + f) * 4 + v) * n1 + kf] = out[v];   // outward
     }
     __syncthreads();
     // phase 3: divergence, DG correction and level-system epilogue
@@ -222,11 +213,12 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
         const dw* Ft = sFt + ((size_t)slot * 4 + v) * N;
         const dw* Gt = sGt + ((size_t)slot * 4 + v) * N;
         dw_acc acc;
+        if (P > 0)
 #pragma unroll
-        for (int m = 0; m < n1; ++m) {
-          acc.add_prod(sD[i][m], Ft[j * n1 + m]);
-          acc.add_prod(sD[j][m], Gt[m * n1 + i]);
-        }
+          for (int m = 0; m < n1; ++m) {
+            acc.add_prod(sD[i][m], Ft[j * n1 + m]);
+            acc.add_prod(sD[j][m], Gt[m * n1 + i]);
+          }
         acc.add_prod(sgL[i], J4[(3 * 4 + v) * n1 + j]);
         acc.add_prod(sgR[i], J4[(1 * 4 + v) * n1 + j]);
         acc.add_prod(sgL[j], J4[(0 * 4 + v) * n1 + i]);

@@ -10,10 +10,15 @@
 // sub-partition, off the FP64 pipe.
 //
 // Same steps and CTA shape as the binary64 kernel: contravariant fluxes of
-// the element's points, the face jumps (common flux minus the extrapolated
-// flux polynomial), the divergence with the DG correction, the level-system
-// epilogue F = R - (q_c(q) - q_c(q_ref)) / (omega dt) + src - S (q_c(q)
-// itself without q_ref), then the block update.  The states hold gauge
+// the element's points, the divergence of each line Dt F + gL F_com(-1) +
+// gR F_com(+1) (the extrapolated part of the DG correction folded into Dt: the
+// separate jump stage it replaces was a quarter of the kernel's instructions
+// and a barrier), the level-system epilogue F = R - (q_c(q) - q_c(q_ref)) /
+// (omega dt) + src - S (q_c(q) itself without q_ref), then the block update.
+// The face launch of a sweep leaves its fluxes as double-words, so neither
+// side converts them.  4096 elements, FP32 blocks (one GB300): P = 1 7.3 -> 6.1
+// us, P = 2 10.5 -> 8.0 us, P = 3 14.7 -> 13.4 us (there the block stream
+// bounds it).  The states hold gauge
 // pressure; with p_ref = 0 (absolute pressure, p ~ 1/(gamma Ma^2) in the
 // momentum flux) the binary64 kernel is used.
 #include "sweep_common.cuh"
@@ -22,7 +27,7 @@ namespace pmg {
 
 template <int P, class W>
 __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
-    int E, double* q, const double* __restrict__ met, const double* __restrict__ Fcom, OpTabW opw, PhysW k,
+    int E, double* q, const double* __restrict__ met, const dw* __restrict__ Fcom, OpTabW opw, PhysW k,
     double inv_odt, const double* __restrict__ src, const double* __restrict__ S, const double* __restrict__ qref,
     const W* __restrict__ Dinv, const double* __restrict__ rs, const double* __restrict__ cs,
     double* __restrict__ werr) {
@@ -34,8 +39,7 @@ __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
   __shared__ Acc sr[EPB][n];
   __shared__ dw sFt[EPB][4][N];
   __shared__ dw sGt[EPB][4][N];
-  __shared__ dw sJ[EPB][4][4][n1];   // [face][var][k]
-  __shared__ dw sD[n1][n1], sgL[n1], sgR[n1], slm[n1], slp[n1];
+  __shared__ dw sD[n1][n1], sgL[n1], sgR[n1];   // Dt, -gL (the fluxes are outward), gR
 
   const int le = threadIdx.x / N, pt = threadIdx.x - le * N;
   const int e = blockIdx.x * EPB + le;
@@ -45,10 +49,10 @@ __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
   W* sDinv = reinterpret_cast<W*>(dsm);
   double* srs = reinterpret_cast<double*>(dsm + PF::dinv_bytes);
   double* scs = srs + EPB * n;
-  double* sFc = scs + EPB * n;   // [v][local element][face][k]
+  dw* sFc = reinterpret_cast<dw*>(scs + EPB * n);   // [v][local element][face][k]
   if (threadIdx.x == 0) {
     const int e0 = blockIdx.x * EPB, ne = min(EPB, E - e0);
-    const unsigned bF = (unsigned)(ne * 4 * n1 * sizeof(double));
+    const unsigned bF = (unsigned)(ne * 4 * n1 * sizeof(dw));
     const unsigned bS = (unsigned)(ne * n * sizeof(double));
     const unsigned bD = PF::blocks ? (unsigned)((size_t)ne * n * n * sizeof(W)) : 0u;
     mbar_init(&mbar[0]);
@@ -76,12 +80,10 @@ __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
 #pragma unroll
     for (int c = 0; c < 5; ++c) mt[c] = __ldg(met + c * plane + gi);
   }
-  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = opw.D[threadIdx.x / n1][threadIdx.x % n1];
+  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = opw.Dt[threadIdx.x / n1][threadIdx.x % n1];
   if (threadIdx.x < n1) {
-    sgL[threadIdx.x] = opw.gL[threadIdx.x];
+    sgL[threadIdx.x] = -opw.gL[threadIdx.x];
     sgR[threadIdx.x] = opw.gR[threadIdx.x];
-    slm[threadIdx.x] = opw.lm[threadIdx.x];
-    slp[threadIdx.x] = opw.lp[threadIdx.x];
   }
 
   dw Q[4], rho = {0.0f, 0.0f};
@@ -89,11 +91,13 @@ __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
 #pragma unroll
     for (int v = 0; v < 4; ++v) Q[v] = dw_from_double(qq[v]);   // gauge p, u, v, T
     rho = (Q[0] + k.p_ref) * rcp(Q[3]);
+    // Cartesian fluxes with the gauge pressure in the momentum rows; at P = 0
+    // the line operator Dt is zero and only the face fluxes remain
+    if (P > 0) {
     const dw a = dw_from_double(mt[0]), b = dw_from_double(mt[1]);
     const dw c = dw_from_double(mt[2]), d = dw_from_double(mt[3]);
     const dw H = k.Cp * Q[3] + half(Q[1] * Q[1] + Q[2] * Q[2]);
     const dw mx = rho * Q[1], my = rho * Q[2];
-    // Cartesian fluxes with the gauge pressure in the momentum rows
     const dw f[4] = {mx, mx * Q[1] + Q[0], mx * Q[2], mx * H};
     const dw g[4] = {my, my * Q[1], my * Q[2] + Q[0], my * H};
 #pragma unroll
@@ -106,26 +110,11 @@ __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
       sFt[le][v][pt] = x.value();
       sGt[le][v][pt] = y.value();
     }
+    }
   }
   __syncthreads();
   const bool okF = mbar_wait0(&mbar[0], k.wait_ns);
   if (!okF) *werr = 1.0;
-  if (active) {
-    for (int it = pt; it < 16 * n1; it += N) {
-      const int f = it / (4 * n1), r = it - f * 4 * n1, v = r / n1, kk = r - v * n1;
-      const bool xi = (f == 1 || f == 3);
-      const bool plus = (f == 1 || f == 2);
-      dw_acc loc;
-#pragma unroll
-      for (int m = 0; m < n1; ++m)
-        loc.add_prod(plus ? slp[m] : slm[m], xi ? sFt[le][v][kk * n1 + m] : sGt[le][v][m * n1 + kk]);
-      const double com = okF ? sFc[((v * EPB + le) * 4 + f) * n1 + kk]
-                             : __ldg(Fcom + v * fplane + ((size_t)e * 4 + f) * n1 + kk);
-      const dw cw = dw_from_double(plus ? com : -com);
-      sJ[le][f][v][kk] = cw - loc.value();
-    }
-  }
-  __syncthreads();
   const bool okS = mbar_wait0(&mbar[1], k.wait_ns);
   if (!okS) *werr = 1.0;
   if (active) {
@@ -154,15 +143,22 @@ __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
       dw_acc acc;
+      if (P > 0)
 #pragma unroll
-      for (int m = 0; m < n1; ++m) {
-        acc.add_prod(sD[i][m], sFt[le][v][j * n1 + m]);
-        acc.add_prod(sD[j][m], sGt[le][v][m * n1 + i]);
+        for (int m = 0; m < n1; ++m) {
+          acc.add_prod(sD[i][m], sFt[le][v][j * n1 + m]);
+          acc.add_prod(sD[j][m], sGt[le][v][m * n1 + i]);
+        }
+      dw com[4];
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const int kk = (f == 1 || f == 3) ? j : i;
+        com[f] = okF ? sFc[((v * EPB + le) * 4 + f) * n1 + kk] : Fcom[v * fplane + ((size_t)e * 4 + f) * n1 + kk];
       }
-      acc.add_prod(sgL[i], sJ[le][3][v][j]);
-      acc.add_prod(sgR[i], sJ[le][1][v][j]);
-      acc.add_prod(sgL[j], sJ[le][0][v][i]);
-      acc.add_prod(sgR[j], sJ[le][2][v][i]);
+      acc.add_prod(sgL[i], com[3]);
+      acc.add_prod(sgR[i], com[1]);
+      acc.add_prod(sgL[j], com[0]);
+      acc.add_prod(sgR[j], com[2]);
       // F = -acc / |J| - qc / (omega dt) + src - S
       dw_acc F;
       F.add_prod(-acc.value(), invJ);
@@ -218,7 +214,7 @@ static void dw_dispatch(const Ctx& c, const LevelDev& L, double* q, double inv_o
   const W* Dinv = (const W*)L.Dinv;
 #define PMG_VDW(PP)                                                                                         \
   volume_apply_dw_kernel<PP, W><<<blocks, threads, VolPrefetch<PP, W>::smem, s>>>(                          \
-      c.E, q, L.met, L.Fcom, L.opw, c.phw, inv_odt, src, S, qref, Dinv, L.rs, L.cs, c.d_scal + 1)
+      c.E, q, L.met, reinterpret_cast<const dw*>(L.Fcom), L.opw, c.phw, inv_odt, src, S, qref, Dinv, L.rs, L.cs, c.d_scal + 1)
   switch (L.P) {
     case 0: PMG_VDW(0); break;
     case 1: PMG_VDW(1); break;

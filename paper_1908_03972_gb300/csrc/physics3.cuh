@@ -83,7 +83,7 @@ __host__ __device__ inline void roe3_flux_jump(const S qm[5], const S qp[5], con
   S w1 = (dp * irho + (1.0 - e2) * un * dun) * iUr2;
   S y0 = (a0 - aun) * w0 + a1 * (e2 * (un * w0 + rc2 * w1));
   S y1 = (a0 - aun) * w1 + a1 * (dun + un * w1);
-  S irCp = irho / ph.Cp;
+  S irCp = irho * ph.inv_Cp;
   S xT = -(1.0 - e2) * un * irCp * y0 + e2 * ph.gm1 * T * y1 + aun * dT;
   S xv[3];
 #pragma unroll

@@ -24,6 +24,7 @@ struct PhysW {
 // Double-word copies of a level's 1D operators (see OpTab).
 struct OpTabW {
   dw D[6][6];
+  dw Dt[6][6];            // D - gL lm^T - gR lp^T
   dw lm[6], lp[6], gL[6], gR[6];
 };
 
@@ -149,7 +150,8 @@ __device__ __forceinline__ void face_roe(const double qm[4], const double qp[4],
     out[2] = fma(pc, ny, dw_to_double(o[2]));
     out[3] = dw_to_double(o[3]);
   } else {
-    roe_flux_jump(qm, qp, dq, pgm, pgp, nx, ny, dS, ph, out);
+    const double n[2] = {nx, ny};
+    roe_jump_d<2>(qm, qp, dq, pgm, pgp, n, dS, ph, out);
   }
 }
 // The double-word face flux left in double-word, the central pressure term

@@ -90,6 +90,8 @@ std::vector<double> element_sizes(const MeshHost& m);
 struct OpTab {
   double D[kMaxP + 1][kMaxP + 1];
   double lm[kMaxP + 1], lp[kMaxP + 1], gL[kMaxP + 1], gR[kMaxP + 1];
+  double Dt[kMaxP + 1][kMaxP + 1];            // D - gL lm^T - gR lp^T
+  double hlm[kMaxP + 1], hlp[kMaxP + 1];      // lm / 2, lp / 2
   double pen;   // BR2 lifting factor eta_f g_R'(1) = 4 (P+1)^2 / 2
 };
 
