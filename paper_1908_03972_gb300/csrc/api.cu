@@ -496,9 +496,8 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
   PMG_CK(cudaMemset(c.src, 0, tot0 * 8));
   c.n_partial = maxblocks;
   PMG_CK(prepare_kernels(c));
-  if (c.dim == 3) {
-    PMG_CK(prepare_kernels3(c));
-  } else {
+  PMG_CK(prepare_assemble(c));
+  if (c.dim == 2) {
     PMG_CK(prepare_residual_kernels(c));
     PMG_CK(prepare_volume_dw_kernels(c));
   }

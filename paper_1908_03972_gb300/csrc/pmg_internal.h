@@ -278,6 +278,7 @@ void launch_volume_apply(const Ctx& c, const LevelDev& L, double* q, double inv_
                          const double* S, const double* qn, int prec, cudaStream_t s);
 void launch_assemble(const Ctx& c, const LevelDev& L, const double* q, const double* d_dtau, double inv_odt,
                      cudaStream_t s);
+cudaError_t prepare_assemble(const Ctx& c);
 void launch_factor(const Ctx& c, LevelDev& L, int level, int prec, int* flag, cudaStream_t s);
 void launch_apply(const Ctx& c, const LevelDev& L, int prec, const double* r, double* x, int accumulate,
                   cudaStream_t s);
@@ -295,7 +296,6 @@ void launch_bsum_update(const Ctx& c, int N, const double* qn, double* const* R,
 void launch_shift_pressure(size_t plane, double delta, double* q, cudaStream_t s);
 void launch_dtau_min(const Ctx& c, double* partial, double* out, cudaStream_t s);
 void launch_grad(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s);
-void launch_assemble_visc(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s);
 void launch_fused_sweep(const Ctx& c, const LevelDev& L, const double* qin, double* qout, double inv_odt,
                         const double* src, const double* S, const double* qref, int prec, cudaStream_t s);
 void launch_loop_controller(LoopState* st, const double* scal, int* sing_flag, double* d_dtau, double* hist_norm,
@@ -310,16 +310,10 @@ void launch_volume3(const Ctx& c, const LevelDev& L, const double* q, double* ou
 void launch_volume_apply3(const Ctx& c, const LevelDev& L, double* q, double inv_odt, const double* src,
                           const double* S, const double* qn, int prec, cudaStream_t s);
 int residual_blocks_for3(int P, int E);
-void launch_assemble3(const Ctx& c, const LevelDev& L, const double* q, const double* d_dtau, double inv_odt,
-                      cudaStream_t s);
-// viscous terms on hexahedra: broken gradients (Gb, 12 planes) and the
-// viscous part of the element blocks (k3_viscous.cu)
+// broken gradients of the viscous terms on hexahedra (Gb, 12 planes)
 void launch_grad3(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s);
-void launch_assemble_visc3(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s);
-cudaError_t prepare_assemble_visc3();
 void launch_apply3(const Ctx& c, const LevelDev& L, int prec, const double* r, double* x, int accumulate,
                    cudaStream_t s);
-cudaError_t prepare_kernels3(const Ctx& c);
 void launch_restrict3(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const XferTab& X, const double* in,
                       double* out, double* out2, double scale, cudaStream_t s);
 void launch_prolong3(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const XferTab& X, const double* qc,
