@@ -97,11 +97,13 @@ static void esdirk_table(Ctx& c, int order) {
 }
 
 static void free_level(LevelDev& L) {
-  double** ptrs[] = {&L.q,     &L.q2, &L.qb, &L.S,  &L.F,  &L.Pd, &L.met,  &L.face,
+  double** ptrs[] = {&L.q,     &L.q2, &L.qb, &L.S,  &L.F,  &L.Pd, &L.met,
                      &L.Fcom,  &L.Dfull, &L.rs, &L.cs, &L.Gb, &L.Qj, &L.fJinv, &L.Cgauge};
   for (double** p : ptrs) { if (*p) cudaFree(*p); *p = nullptr; }
   int** iptrs[] = {&L.d_toff, &L.d_tlayer, &L.d_telems, &L.d_tlnbr};
   for (int** p : iptrs) { if (*p) cudaFree(*p); *p = nullptr; }
+  L.face = nullptr;   // face, metW and faceW lie in met's allocation
+  L.metW = L.faceW = nullptr;
   if (L.Dinv) cudaFree(L.Dinv);
   L.Dinv = nullptr;
 }
@@ -427,7 +429,7 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
     }
     size_t nn2 = (size_t)c.E * L.n * L.n;
     if (dalloc(&L.q, L.tot) || dalloc(&L.qb, L.tot) || dalloc(&L.S, L.tot) || dalloc(&L.F, L.tot) ||
-        dalloc(&L.Pd, L.tot) || dalloc(&L.met, geo[l].met.size()) || dalloc(&L.face, geo[l].face.size()) ||
+        dalloc(&L.Pd, L.tot) ||
         dalloc(&L.Fcom, (size_t)c.nv * c.E * c.nfc * L.NF) || dalloc(&L.Dfull, nn2) ||
         cudaMalloc(&L.Dinv, nn2 * wbytes) || dalloc(&L.rs, (size_t)c.E * L.n) || dalloc(&L.cs, (size_t)c.E * L.n))
       return fail(PMG_ENOMEM, "device allocation failed for level data");
@@ -471,8 +473,27 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
     }
     PMG_CK(cudaMemset(L.S, 0, L.tot * 8));
     PMG_CK(cudaMemset(L.q, 0, L.tot * 8));
-    PMG_CK(cudaMemcpy(L.met, geo[l].met.data(), geo[l].met.size() * 8, cudaMemcpyHostToDevice));
-    PMG_CK(cudaMemcpy(L.face, geo[l].face.data(), geo[l].face.size() * 8, cudaMemcpyHostToDevice));
+    {
+      // metrics and face geometry, and (2D) both in double-word for the
+      // sweeps, in one buffer and one copy
+      const size_t nm = geo[l].met.size(), nfc = geo[l].face.size(), nb = nm + nfc;
+      const bool words = c.dim == 2;
+      std::vector<double> buf(words ? 2 * nb : nb);
+      std::copy(geo[l].met.begin(), geo[l].met.end(), buf.begin());
+      std::copy(geo[l].face.begin(), geo[l].face.end(), buf.begin() + nm);
+      if (words)
+        for (size_t i = 0; i < nb; ++i) {
+          const dw w = dw_const(buf[i]);
+          memcpy(&buf[nb + i], &w, sizeof(w));
+        }
+      if (dalloc(&L.met, buf.size())) return fail(PMG_ENOMEM, "device allocation failed for level data");
+      PMG_CK(cudaMemcpy(L.met, buf.data(), buf.size() * 8, cudaMemcpyHostToDevice));
+      L.face = L.met + nm;
+      if (words) {
+        L.metW = reinterpret_cast<dw*>(L.met + nb);
+        L.faceW = L.metW + nm;
+      }
+    }
     c.xy_host[l] = geo[l].xy;
     maxblocks = std::max(maxblocks, c.dim == 3 ? residual_blocks_for3(L.P, c.E) : residual_blocks_for(L.P, c.E));
   }

@@ -67,6 +67,51 @@ __device__ __forceinline__ dw operator*(dw x, dw y) {
   return fast_two_sum(ch, cl);
 }
 
+// Sums of products with one renormalisation at the end (Dot2): the high
+// products exactly (2Prod), their sum exactly (2Sum), every low-order term in
+// one word.  a b + c takes 15 operations (18 as a product and a sum), a b + c d
+// 19 (25), and the chain between renormalisations is shorter.
+__device__ __forceinline__ dw mul_add(dw a, dw b, dw c) {   // a b + c
+  const float ph = __fmul_rn(a.h, b.h);
+  float pl = __fmaf_rn(a.h, b.h, -ph);
+  pl = __fmaf_rn(a.h, b.l, pl);
+  pl = __fmaf_rn(a.l, b.h, pl);
+  const dw s = two_sum(ph, c.h);
+  return fast_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(pl, c.l)));
+}
+__device__ __forceinline__ dw dot2(dw a, dw b, dw c, dw d) {   // a b + c d
+  const float ph = __fmul_rn(a.h, b.h), rh = __fmul_rn(c.h, d.h);
+  float pl = __fmaf_rn(a.h, b.h, -ph), rl = __fmaf_rn(c.h, d.h, -rh);
+  pl = __fmaf_rn(a.h, b.l, pl);
+  rl = __fmaf_rn(c.h, d.l, rl);
+  pl = __fmaf_rn(a.l, b.h, pl);
+  rl = __fmaf_rn(c.l, d.h, rl);
+  const dw s = two_sum(ph, rh);
+  return fast_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(pl, rl)));
+}
+__device__ __forceinline__ dw dot2_add(dw a, dw b, dw c, dw d, dw e) {   // a b + c d + e
+  const float ph = __fmul_rn(a.h, b.h), rh = __fmul_rn(c.h, d.h);
+  float pl = __fmaf_rn(a.h, b.h, -ph), rl = __fmaf_rn(c.h, d.h, -rh);
+  pl = __fmaf_rn(a.h, b.l, pl);
+  rl = __fmaf_rn(c.h, d.l, rl);
+  pl = __fmaf_rn(a.l, b.h, pl);
+  rl = __fmaf_rn(c.l, d.h, rl);
+  const dw s = two_sum(ph, rh), t = two_sum(s.h, e.h);
+  return fast_two_sum(t.h, __fadd_rn(__fadd_rn(s.l, t.l), __fadd_rn(__fadd_rn(pl, rl), e.l)));
+}
+__device__ __forceinline__ dw dot3(dw a, dw b, dw c, dw d, dw e, dw f) {   // a b + c d + e f
+  const float ph = __fmul_rn(a.h, b.h), rh = __fmul_rn(c.h, d.h), th = __fmul_rn(e.h, f.h);
+  float pl = __fmaf_rn(a.h, b.h, -ph), rl = __fmaf_rn(c.h, d.h, -rh), tl = __fmaf_rn(e.h, f.h, -th);
+  pl = __fmaf_rn(a.h, b.l, pl);
+  rl = __fmaf_rn(c.h, d.l, rl);
+  tl = __fmaf_rn(e.h, f.l, tl);
+  pl = __fmaf_rn(a.l, b.h, pl);
+  rl = __fmaf_rn(c.l, d.h, rl);
+  tl = __fmaf_rn(e.l, f.h, tl);
+  const dw s = two_sum(ph, rh), t = two_sum(s.h, th);
+  return fast_two_sum(t.h, __fadd_rn(__fadd_rn(s.l, t.l), __fadd_rn(__fadd_rn(pl, rl), tl)));
+}
+
 // x * 2^k is exact: scale both parts.
 __device__ __forceinline__ dw scale2(dw x, float pow2) { return {__fmul_rn(x.h, pow2), __fmul_rn(x.l, pow2)}; }
 

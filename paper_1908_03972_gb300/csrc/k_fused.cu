@@ -151,14 +151,11 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_kernel(
           sp[v] = s;
         }
       }
-      double qm[4], qp[4], dq[4];
+      double dq[4];
 #pragma unroll
-      for (int v = 0; v < 4; ++v) { qm[v] = ref[v] + sm[v]; qp[v] = ref[v] + sp[v]; dq[v] = sp[v] - sm[v]; }
-      const double pgm = qm[0], pgp = qp[0];
-      qm[0] += ph.p_ref;
-      qp[0] += ph.p_ref;
+      for (int v = 0; v < 4; ++v) dq[v] = sp[v] - sm[v];
       double out[4];
-      face_roe<DWF>(qm, qp, dq, pgm, pgp, gx, gy, gS, ph, phw, out);
+      face_roe<DWF>(ref, sm, sp, dq, gx, gy, gS, ph, phw, out);
 #pragma unroll
       for (int v = 0; v < 4; ++v) sJ[le][f][v][k] = out[v];   // outward
     }
@@ -243,8 +240,8 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_kernel(
 // still formed in binary64 relative to the element's first point.
 template <int P, class W>
 __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
-    int E, const double* __restrict__ qin, double* __restrict__ qout, const double* __restrict__ met,
-    const double* __restrict__ face, const int* __restrict__ nbr, OpTabW opw, OpTab op, PhysW k, double p_ref,
+    int E, const double* __restrict__ qin, double* __restrict__ qout, const dw* __restrict__ met,
+    const dw* __restrict__ face, const int* __restrict__ nbr, OpTabW opw, OpTab op, PhysW k,
     double inv_odt, const double* __restrict__ S, const double* __restrict__ qref, const W* __restrict__ Dinv,
     const double* __restrict__ rs, const double* __restrict__ cs, double* __restrict__ werr) {
   constexpr int n1 = P + 1, N = n1 * n1, n = 4 * N, EPB = FusedEPB<P>::value, FP = 4 * n1;
@@ -277,8 +274,8 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
   const bool act = le < EPB && e < E;
   const bool own = act && t < N;
   const int f = t / n1, kf = t - f * n1;
-  double nq[4][n1], gx = 0.0, gy = 0.0, gS = 0.0, qq[4] = {0, 0, 0, 0}, qo[4] = {0, 0, 0, 0};
-  double Sv[4] = {0, 0, 0, 0}, mt[5] = {0, 0, 0, 0, 0};
+  double nq[4][n1], qq[4] = {0, 0, 0, 0}, qo[4] = {0, 0, 0, 0}, Sv[4] = {0, 0, 0, 0};
+  dw gx = {}, gy = {}, gS = {}, mt[5] = {};
   int fn = 0;   // neighbour's face
   if (act) {
     const int en = __ldg(nbr + (e * 4 + f) * 3 + 0);
@@ -291,10 +288,10 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
     for (int v = 0; v < 4; ++v)
 #pragma unroll
       for (int m = 0; m < n1; ++m) nq[v][m] = __ldg(base + v * plane + m * stride);
-    const double* g = face + (((size_t)e * 4 + f) * n1 + kf) * 3;
-    gx = __ldg(g);
-    gy = __ldg(g + 1);
-    gS = __ldg(g + 2);
+    const dw* g = face + (((size_t)e * 4 + f) * n1 + kf) * 3;
+    gx = g[0];
+    gy = g[1];
+    gS = g[2];
   }
   if (own) {
     const size_t gi = (size_t)e * N + t;
@@ -305,7 +302,7 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
       if (S) Sv[v] = -__ldg(S + v * plane + gi);
     }
 #pragma unroll
-    for (int c = 0; c < 5; ++c) mt[c] = __ldg(met + c * plane + gi);
+    for (int c = 0; c < 5; ++c) mt[c] = met[c * plane + gi];
   }
   if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = opw.Dt[threadIdx.x / n1][threadIdx.x % n1];
   if (threadIdx.x < n1) {
@@ -325,21 +322,14 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
     }
     rho = (Q[0] + k.p_ref) * rcp(Q[3]);
     if (P > 0) {   // at P = 0 the line operator Dt is zero
-      const dw a = dw_from_double(mt[0]), b = dw_from_double(mt[1]);
-      const dw c = dw_from_double(mt[2]), d = dw_from_double(mt[3]);
-      const dw H = k.Cp * Q[3] + half(Q[1] * Q[1] + Q[2] * Q[2]);
+      const dw H = mul_add(k.Cp, Q[3], half(dot2(Q[1], Q[1], Q[2], Q[2])));
       const dw mx = rho * Q[1], my = rho * Q[2];
-      const dw fx[4] = {mx, mx * Q[1] + Q[0], mx * Q[2], mx * H};
-      const dw gy4[4] = {my, my * Q[1], my * Q[2] + Q[0], my * H};
+      const dw fx[4] = {mx, mul_add(mx, Q[1], Q[0]), mx * Q[2], mx * H};
+      const dw gy4[4] = {my, fx[2], mul_add(my, Q[2], Q[0]), my * H};
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
-        dw_acc x, y;
-        x.add_prod(a, fx[v]);
-        x.add_prod(b, gy4[v]);
-        y.add_prod(c, fx[v]);
-        y.add_prod(d, gy4[v]);
-        sFt[le][v][t] = x.value();
-        sGt[le][v][t] = y.value();
+        sFt[le][v][t] = dot2(mt[0], fx[v], mt[1], gy4[v]);
+        sGt[le][v][t] = dot2(mt[2], fx[v], mt[3], gy4[v]);
       }
     }
   }
@@ -354,26 +344,24 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
       double a = 0.0, b = 0.0;
+      if (P == 0) {   // one point of weight 1, which is the reference
+        a = v == 0 || v == 3 ? 0.0 : sq[le][v][0];
+        b = nq[v][0] - ref[v];
+      } else {
 #pragma unroll
-      for (int m = 0; m < n1; ++m) {
-        a = fma(plus ? slp[m] : slm[m], sq[le][v][eta ? m * n1 + kf : kf * n1 + m] - ref[v], a);
-        b = fma(pn ? slp[m] : slm[m], nq[v][m] - ref[v], b);
+        for (int m = 0; m < n1; ++m) {
+          a = fma(plus ? slp[m] : slm[m], sq[le][v][eta ? m * n1 + kf : kf * n1 + m] - ref[v], a);
+          b = fma(pn ? slp[m] : slm[m], nq[v][m] - ref[v], b);
+        }
       }
       sm[v] = a;
       sp[v] = b;
     }
-    double qm[4], qp[4], dq[4];
+    double dq[4];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      qm[v] = ref[v] + sm[v];
-      qp[v] = ref[v] + sp[v];
-      dq[v] = sp[v] - sm[v];
-    }
-    const double pgm = qm[0], pgp = qp[0];
-    qm[0] += p_ref;
-    qp[0] += p_ref;
+    for (int v = 0; v < 4; ++v) dq[v] = P == 0 && (v == 0 || v == 3) ? sp[v] : sp[v] - sm[v];
     dw out[4];
-    face_roe_dw(qm, qp, dq, pgm, pgp, gx, gy, gS, k, out);
+    face_roe_dw(ref[0], ref[3], sm, dq, gx, gy, gS, k, out);
 #pragma unroll
     for (int v = 0; v < 4; ++v) sJ[le][f][v][kf] = out[v];   // outward
   }
@@ -390,17 +378,17 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
       for (int v = 0; v < 4; ++v) Qo[v] = dw_from_double(qo[v]);
       const dw rhoo = (Qo[0] + k.p_ref) * rcp(Qo[3]);
       qc[0] = rho - rhoo;
-      qc[1] = rho * Q[1] - rhoo * Qo[1];
-      qc[2] = rho * Q[2] - rhoo * Qo[2];
-      qc[3] = (Q[0] - Qo[0]) * k.inv_gm1 +
-              half(rho * (Q[1] * Q[1] + Q[2] * Q[2]) - rhoo * (Qo[1] * Qo[1] + Qo[2] * Qo[2]));
+      qc[1] = dot2(rho, Q[1], -rhoo, Qo[1]);
+      qc[2] = dot2(rho, Q[2], -rhoo, Qo[2]);
+      qc[3] = mul_add(Q[0] - Qo[0], k.inv_gm1,
+                      half(dot2(rho, dot2(Q[1], Q[1], Q[2], Q[2]), -rhoo, dot2(Qo[1], Qo[1], Qo[2], Qo[2]))));
     } else {
       qc[0] = rho;
       qc[1] = rho * Q[1];
       qc[2] = rho * Q[2];
       qc[3] = rho * (Q[3] * k.inv_gm1 + half(Q[1] * Q[1] + Q[2] * Q[2]));
     }
-    const dw invJ = dw_from_double(mt[4]);
+    const dw ninvJ = -mt[4];
     const dw nodt = dw_from_double(-inv_odt);
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
@@ -415,12 +403,10 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
       acc.add_prod(sgR[i], sJ[le][1][v][j]);
       acc.add_prod(sgL[j], sJ[le][0][v][i]);
       acc.add_prod(sgR[j], sJ[le][2][v][i]);
-      dw_acc F;   // -acc / |J| - qc / (omega dt) - S
-      F.add_prod(-acc.value(), invJ);
-      F.add_prod(qc[v], nodt);
-      F.add(dw_from_double(Sv[v]));
+      // -acc / |J| - qc / (omega dt) - S
+      const dw F = dot2_add(acc.value(), ninvJ, qc[v], nodt, dw_from_double(Sv[v]));
       const int row = v * N + t;
-      sr[le][row] = scaled_in_dw<W>(F.value(), ok ? srs[le * n + row] : rs[(size_t)e * n + row]);
+      sr[le][row] = scaled_in_dw<W>(F, ok ? srs[le * n + row] : rs[(size_t)e * n + row]);
     }
   }
   __syncthreads();
@@ -460,7 +446,7 @@ static void fused_launch(const Ctx& c, const LevelDev& L, const double* qin, dou
   if (dwf && c.ph.p_ref != 0.0 && !src) {   // gauge storage: the double-word sweep
 #define PMG_FUSED_DW(WT)                                                                         \
   fused_sweep_dw_kernel<P, WT><<<blocks, threads, fused_smem<P, WT>(), s>>>(                       \
-      c.E, qin, qout, L.met, L.face, nbr, L.opw, L.op, c.phw, c.ph.p_ref, inv_odt, S, qref,        \
+      c.E, qin, qout, L.metW, L.faceW, nbr, L.opw, L.op, c.phw, inv_odt, S, qref,                  \
       (const WT*)L.Dinv, L.rs, L.cs, c.d_scal + 1)
     if (prec == PMG_PREC_FP64) PMG_FUSED_DW(double);
     else if (prec == PMG_PREC_BF16R) PMG_FUSED_DW(__nv_bfloat16);

@@ -56,6 +56,10 @@ __device__ __forceinline__ void line_trace(const double* __restrict__ q, size_t 
   const int stride = eta ? n1 : 1;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
+    if (P == 0) {   // one point: the weight is 1
+      out[v] = __ldg(base + v * plane) - ref[v];
+      continue;
+    }
     double s = 0.0;
 #pragma unroll
     for (int m = 0; m < n1; ++m) s = fma(plus ? lp[m] : lm[m], __ldg(base + v * plane + m * stride) - ref[v], s);
@@ -86,6 +90,7 @@ template <int P, bool VISC, bool DWF, bool OUTDW>
 __global__ void __launch_bounds__(256) face_flux_kernel(const int* __restrict__ faces, int n_faces, int E,
                                                         const double* __restrict__ q,
                                                         const double* __restrict__ face,
+                                                        const dw* __restrict__ faceW,
                                                         double* __restrict__ Fcom, OpTab op, Phys ph, PhysW phw,
                                                         const double* __restrict__ Gb,
                                                         const double* __restrict__ fJinv,
@@ -127,22 +132,16 @@ __global__ void __launch_bounds__(256) face_flux_kernel(const int* __restrict__ 
       sp[2] = fma(-2.0 * un, ny, sm[2]);
     }
   }
-  double qm[4], qp[4], dq[4];
+  double dq[4];
 #pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    qm[v] = ref[v] + sm[v];
-    qp[v] = ref[v] + sp[v];
-    dq[v] = sp[v] - sm[v];
-  }
-  const double pgm = qm[0], pgp = qp[0];   // gauge pressures for the momentum fluxes
-  qm[0] += ph.p_ref;   // absolute pressure for the averaged state and rho
-  qp[0] += ph.p_ref;
+  for (int v = 0; v < 4; ++v) dq[v] = sp[v] - sm[v];
   const size_t fplane = (size_t)E * 4 * n1;
   const size_t iL = ((size_t)eL * 4 + fL) * n1 + k;
   const size_t iR = bnd ? iL : ((size_t)eR * 4 + fR) * n1 + kR;
   if (OUTDW) {
     dw o[4];
-    face_roe_dw(qm, qp, dq, pgm, pgp, nx, ny, dS, phw, o);
+    const dw* gw = faceW + (((size_t)eL * 4 + fL) * n1 + k) * 3;
+    face_roe_dw(ref[0], ref[3], sm, dq, gw[0], gw[1], gw[2], phw, o);
     dw* Fw = reinterpret_cast<dw*>(Fcom);
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
@@ -152,7 +151,7 @@ __global__ void __launch_bounds__(256) face_flux_kernel(const int* __restrict__ 
     return;
   }
   double out[4];
-  face_roe<DWF>(qm, qp, dq, pgm, pgp, nx, ny, dS, ph, phw, out);
+  face_roe<DWF>(ref, sm, sp, dq, nx, ny, dS, ph, phw, out);
   if (VISC) {
     // common gradient: mean of the two broken-gradient traces plus the BR2
     // liftings r^- + r^+ = pen (q_com - q^-) (1/|J|^- + 1/|J|^+) n dS, with
@@ -170,7 +169,7 @@ __global__ void __launch_bounds__(256) face_flux_kernel(const int* __restrict__ 
       grad_trace<P>(Gb, plane, bnd ? eL : eR, bnd ? fL : fR, bnd ? k : kR, op.hlm, op.hlp, gc);
     }
     double fv[4], gv[4];
-    viscous_flux(0.5 * (qm[1] + qp[1]), 0.5 * (qm[2] + qp[2]), gc, ph, fv, gv);
+    viscous_flux(fma(0.5, dq[1], sm[1]), fma(0.5, dq[2], sm[2]), gc, ph, fv, gv);
     const int nv = (bnd && fR != PMG_BC_FARFIELD) ? 3 : 4;   // walls: no viscous energy flux
 #pragma unroll
     for (int v = 1; v < 4; ++v)
@@ -482,7 +481,7 @@ void launch_face_flux(const Ctx& c, const LevelDev& L, const double* q, cudaStre
   if (visc) launch_grad(c, L, q, s);
   const bool outdw = sweep && volume_dw_applies(c);
 #define PMG_FACE_V(PP, V, D, O)                                                                              \
-  face_flux_kernel<PP, V, D, O><<<blocks, threads, 0, s>>>(c.d_faces, c.n_faces, c.E, q, L.face, L.Fcom, L.op, \
+  face_flux_kernel<PP, V, D, O><<<blocks, threads, 0, s>>>(c.d_faces, c.n_faces, c.E, q, L.face, L.faceW, L.Fcom, L.op, \
                                                         c.ph, c.phw, V ? L.Gb : nullptr,                    \
                                                         V ? L.fJinv : nullptr, V ? L.Qj : nullptr)
 #define PMG_FACE(PP)                                   \

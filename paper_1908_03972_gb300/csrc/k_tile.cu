@@ -40,8 +40,8 @@ template <int P, class W>
 __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
     const int* __restrict__ toff, const int* __restrict__ tlayer, const int* __restrict__ telems,
     const int* __restrict__ tlnbr, int depth, int nsweep, int E, const double* __restrict__ qin,
-    double* __restrict__ qout, const double* __restrict__ met, const double* __restrict__ face,
-    const int* __restrict__ nbr, OpTabW opw, OpTab op, PhysW k, double p_ref, double inv_odt,
+    double* __restrict__ qout, const dw* __restrict__ met, const dw* __restrict__ face,
+    const int* __restrict__ nbr, OpTabW opw, OpTab op, PhysW k, double inv_odt,
     const double* __restrict__ S, const double* __restrict__ qref, const W* __restrict__ Dinv,
     const double* __restrict__ rs, const double* __restrict__ cs) {
   using L = TileLayout<P, W>;
@@ -55,9 +55,9 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
   double* srs = reinterpret_cast<double*>(dsm);
   double* scs = srs + (size_t)M * n;
   double* sq0 = scs + (size_t)M * n;                 // [2][M][4][N]
-  double* smt = sq0 + (size_t)2 * M * 4 * N;         // [M][5][N]
-  double* sfg = smt + (size_t)M * 5 * N;             // [M][FP][3]
-  double* sqo = sfg + (size_t)M * FP * 3;            // [M][4][N]
+  dw* smt = reinterpret_cast<dw*>(sq0 + (size_t)2 * M * 4 * N);   // [M][5][N]
+  dw* sfg = smt + (size_t)M * 5 * N;                 // [M][FP][3]
+  double* sqo = reinterpret_cast<double*>(sfg + (size_t)M * FP * 3);   // [M][4][N]
   double* sSv = sqo + (size_t)M * 4 * N;             // [M][4][N]
   dw* sFt = reinterpret_cast<dw*>(sSv + (size_t)M * 4 * N);   // [M][4][N]
   dw* sGt = sFt + (size_t)M * 4 * N;
@@ -93,9 +93,9 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
   const int f = tf / n1, kf = tf - f * n1;
   if (mine) {
     const int e = telems[t0 + slot];
-    const double* g = face + (((size_t)e * 4 + f) * n1 + kf) * 3;
+    const dw* g = face + (((size_t)e * 4 + f) * n1 + kf) * 3;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) sfg[((size_t)slot * FP + tf) * 3 + c] = __ldg(g + c);
+    for (int c = 0; c < 3; ++c) sfg[((size_t)slot * FP + tf) * 3 + c] = g[c];
     if (own) {
       const size_t gi = (size_t)e * N + tf;
 #pragma unroll
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
         sSv[((size_t)slot * 4 + v) * N + tf] = S ? -__ldg(S + v * plane + gi) : 0.0;
       }
 #pragma unroll
-      for (int c = 0; c < 5; ++c) smt[((size_t)slot * 5 + c) * N + tf] = __ldg(met + c * plane + gi);
+      for (int c = 0; c < 5; ++c) smt[((size_t)slot * 5 + c) * N + tf] = met[c * plane + gi];
     }
   }
   if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = opw.Dt[threadIdx.x / n1][threadIdx.x % n1];
@@ -128,22 +128,17 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
 #pragma unroll
       for (int v = 0; v < 4; ++v) Q[v] = dw_from_double(sqA[((size_t)slot * 4 + v) * N + tf]);
       rho = (Q[0] + k.p_ref) * rcp(Q[3]);
-      const double* mt = smt + (size_t)slot * 5 * N;
-      const dw a = dw_from_double(mt[0 * N + tf]), b = dw_from_double(mt[1 * N + tf]);
-      const dw c = dw_from_double(mt[2 * N + tf]), d = dw_from_double(mt[3 * N + tf]);
-      const dw H = k.Cp * Q[3] + half(Q[1] * Q[1] + Q[2] * Q[2]);
-      const dw mx = rho * Q[1], my = rho * Q[2];
-      const dw fx[4] = {mx, mx * Q[1] + Q[0], mx * Q[2], mx * H};
-      const dw gy4[4] = {my, my * Q[1], my * Q[2] + Q[0], my * H};
+      if (P > 0) {   // at P = 0 the line operator Dt is zero
+        const dw* mt = smt + (size_t)slot * 5 * N;
+        const dw H = mul_add(k.Cp, Q[3], half(dot2(Q[1], Q[1], Q[2], Q[2])));
+        const dw mx = rho * Q[1], my = rho * Q[2];
+        const dw fx[4] = {mx, mul_add(mx, Q[1], Q[0]), mx * Q[2], mx * H};
+        const dw gy4[4] = {my, fx[2], mul_add(my, Q[2], Q[0]), my * H};
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        dw_acc x, y;
-        x.add_prod(a, fx[v]);
-        x.add_prod(b, gy4[v]);
-        y.add_prod(c, fx[v]);
-        y.add_prod(d, gy4[v]);
-        sFt[((size_t)slot * 4 + v) * N + tf] = x.value();
-        sGt[((size_t)slot * 4 + v) * N + tf] = y.value();
+        for (int v = 0; v < 4; ++v) {
+          sFt[((size_t)slot * 4 + v) * N + tf] = dot2(mt[0 * N + tf], fx[v], mt[1 * N + tf], gy4[v]);
+          sGt[((size_t)slot * 4 + v) * N + tf] = dot2(mt[2 * N + tf], fx[v], mt[3 * N + tf], gy4[v]);
+        }
       }
     }
     __syncthreads();
@@ -160,27 +155,25 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         double a = 0.0, b = 0.0;
+        if (P == 0) {   // one point of weight 1, which is the reference
+          a = v == 0 || v == 3 ? 0.0 : sqe[v];
+          b = sqn[v] - ref[v];
+        } else {
 #pragma unroll
-        for (int m = 0; m < n1; ++m) {
-          a = fma(plus ? slp[m] : slm[m], sqe[v * N + (eta ? m * n1 + kf : kf * n1 + m)] - ref[v], a);
-          b = fma(pn ? slp[m] : slm[m], sqn[v * N + (etan ? m * n1 + kn : kn * n1 + m)] - ref[v], b);
+          for (int m = 0; m < n1; ++m) {
+            a = fma(plus ? slp[m] : slm[m], sqe[v * N + (eta ? m * n1 + kf : kf * n1 + m)] - ref[v], a);
+            b = fma(pn ? slp[m] : slm[m], sqn[v * N + (etan ? m * n1 + kn : kn * n1 + m)] - ref[v], b);
+          }
         }
         sm[v] = a;
         sp[v] = b;
       }
-      double qm[4], qp[4], dq[4];
+      double dq[4];
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        qm[v] = ref[v] + sm[v];
-        qp[v] = ref[v] + sp[v];
-        dq[v] = sp[v] - sm[v];
-      }
-      const double pgm = qm[0], pgp = qp[0];
-      qm[0] += p_ref;
-      qp[0] += p_ref;
-      const double* g = sfg + ((size_t)slot * FP + tf) * 3;
+      for (int v = 0; v < 4; ++v) dq[v] = P == 0 && (v == 0 || v == 3) ? sp[v] : sp[v] - sm[v];
+      const dw* g = sfg + ((size_t)slot * FP + tf) * 3;
       dw out[4];
-      face_roe_dw(qm, qp, dq, pgm, pgp, g[0], g[1], g[2], k, out);
+      face_roe_dw(ref[0], ref[3], sm, dq, g[0], g[1], g[2], k, out);
 #pragma unroll
       for (int v = 0; v < 4; ++v) sJ[(((size_t)slot * 4 + f) * 4 + v) * n1 + kf] = out[v];   // outward
     }
@@ -195,17 +188,17 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
         for (int v = 0; v < 4; ++v) Qo[v] = dw_from_double(sqo[((size_t)slot * 4 + v) * N + tf]);
         const dw rhoo = (Qo[0] + k.p_ref) * rcp(Qo[3]);
         qc[0] = rho - rhoo;
-        qc[1] = rho * Q[1] - rhoo * Qo[1];
-        qc[2] = rho * Q[2] - rhoo * Qo[2];
-        qc[3] = (Q[0] - Qo[0]) * k.inv_gm1 +
-                half(rho * (Q[1] * Q[1] + Q[2] * Q[2]) - rhoo * (Qo[1] * Qo[1] + Qo[2] * Qo[2]));
+        qc[1] = dot2(rho, Q[1], -rhoo, Qo[1]);
+        qc[2] = dot2(rho, Q[2], -rhoo, Qo[2]);
+        qc[3] = mul_add(Q[0] - Qo[0], k.inv_gm1,
+                        half(dot2(rho, dot2(Q[1], Q[1], Q[2], Q[2]), -rhoo, dot2(Qo[1], Qo[1], Qo[2], Qo[2]))));
       } else {
         qc[0] = rho;
         qc[1] = rho * Q[1];
         qc[2] = rho * Q[2];
         qc[3] = rho * (Q[3] * k.inv_gm1 + half(Q[1] * Q[1] + Q[2] * Q[2]));
       }
-      const dw invJ = dw_from_double(smt[((size_t)slot * 5 + 4) * N + tf]);
+      const dw ninvJ = -smt[((size_t)slot * 5 + 4) * N + tf];
       const dw nodt = dw_from_double(-inv_odt);
       const dw* J4 = sJ + (size_t)slot * 16 * n1;
 #pragma unroll
@@ -223,12 +216,9 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
         acc.add_prod(sgR[i], J4[(1 * 4 + v) * n1 + j]);
         acc.add_prod(sgL[j], J4[(0 * 4 + v) * n1 + i]);
         acc.add_prod(sgR[j], J4[(2 * 4 + v) * n1 + i]);
-        dw_acc F;
-        F.add_prod(-acc.value(), invJ);
-        F.add_prod(qc[v], nodt);
-        F.add(dw_from_double(sSv[((size_t)slot * 4 + v) * N + tf]));
+        const dw F = dot2_add(acc.value(), ninvJ, qc[v], nodt, dw_from_double(sSv[((size_t)slot * 4 + v) * N + tf]));
         const int row = v * N + tf;
-        sr[(size_t)slot * n + row] = scaled_in_dw<W>(F.value(), srs[(size_t)slot * n + row]);
+        sr[(size_t)slot * n + row] = scaled_in_dw<W>(F, srs[(size_t)slot * n + row]);
       }
     }
     __syncthreads();
@@ -267,8 +257,8 @@ static void tile_launch(const Ctx& c, const LevelDev& L, const double* qin, doub
   using Lay = TileLayout<P, W>;
   const int threads = (L.tile_M * Lay::FP + 31) / 32 * 32;
   tile_sweep_dw_kernel<P, W><<<L.n_tiles, threads, Lay::bytes(L.tile_M), s>>>(
-      L.d_toff, L.d_tlayer, L.d_telems, L.d_tlnbr, L.tile_depth, nsweep, c.E, qin, qout, L.met, L.face,
-      c.d_faces + 5 * c.n_faces, L.opw, L.op, c.phw, c.ph.p_ref, inv_odt, S, qref, (const W*)L.Dinv, L.rs, L.cs);
+      L.d_toff, L.d_tlayer, L.d_telems, L.d_tlnbr, L.tile_depth, nsweep, c.E, qin, qout, L.metW, L.faceW,
+      c.d_faces + 5 * c.n_faces, L.opw, L.op, c.phw, inv_odt, S, qref, (const W*)L.Dinv, L.rs, L.cs);
 }
 
 // One launch of nsweep (<= the tile depth) sweeps of a tiled level.

@@ -27,7 +27,7 @@ namespace pmg {
 
 template <int P, class W>
 __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
-    int E, double* q, const double* __restrict__ met, const dw* __restrict__ Fcom, OpTabW opw, PhysW k,
+    int E, double* q, const dw* __restrict__ met, const dw* __restrict__ Fcom, OpTabW opw, PhysW k,
     double inv_odt, const double* __restrict__ src, const double* __restrict__ S, const double* __restrict__ qref,
     const W* __restrict__ Dinv, const double* __restrict__ rs, const double* __restrict__ cs,
     double* __restrict__ werr) {
@@ -68,17 +68,18 @@ __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
   }
   const size_t gi = (size_t)e * N + pt;
   // Sv: src - S of the epilogue
-  double qq[4] = {0, 0, 0, 0}, qo[4] = {0, 0, 0, 0}, Sv[4] = {0, 0, 0, 0}, mt[5] = {0, 0, 0, 0, 0};
+  double qq[4] = {0, 0, 0, 0}, qo[4] = {0, 0, 0, 0}, Sv[4] = {0, 0, 0, 0};
+  dw mt[5] = {};
   if (active) {
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
       qq[v] = q[v * plane + gi];
       if (qref) qo[v] = __ldg(qref + v * plane + gi);
       if (src) Sv[v] = __ldg(src + v * plane + gi);
-      if (S) Sv[v] -= __ldg(S + v * plane + gi);
+      if (S) Sv[v] = src ? Sv[v] - __ldg(S + v * plane + gi) : -__ldg(S + v * plane + gi);
     }
 #pragma unroll
-    for (int c = 0; c < 5; ++c) mt[c] = __ldg(met + c * plane + gi);
+    for (int c = 0; c < 5; ++c) mt[c] = met[c * plane + gi];
   }
   if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = opw.Dt[threadIdx.x / n1][threadIdx.x % n1];
   if (threadIdx.x < n1) {
@@ -94,22 +95,15 @@ __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
     // Cartesian fluxes with the gauge pressure in the momentum rows; at P = 0
     // the line operator Dt is zero and only the face fluxes remain
     if (P > 0) {
-    const dw a = dw_from_double(mt[0]), b = dw_from_double(mt[1]);
-    const dw c = dw_from_double(mt[2]), d = dw_from_double(mt[3]);
-    const dw H = k.Cp * Q[3] + half(Q[1] * Q[1] + Q[2] * Q[2]);
-    const dw mx = rho * Q[1], my = rho * Q[2];
-    const dw f[4] = {mx, mx * Q[1] + Q[0], mx * Q[2], mx * H};
-    const dw g[4] = {my, my * Q[1], my * Q[2] + Q[0], my * H};
+      const dw H = mul_add(k.Cp, Q[3], half(dot2(Q[1], Q[1], Q[2], Q[2])));
+      const dw mx = rho * Q[1], my = rho * Q[2];
+      const dw f[4] = {mx, mul_add(mx, Q[1], Q[0]), mx * Q[2], mx * H};
+      const dw g[4] = {my, f[2], mul_add(my, Q[2], Q[0]), my * H};
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      dw_acc x, y;
-      x.add_prod(a, f[v]);
-      x.add_prod(b, g[v]);
-      y.add_prod(c, f[v]);
-      y.add_prod(d, g[v]);
-      sFt[le][v][pt] = x.value();
-      sGt[le][v][pt] = y.value();
-    }
+      for (int v = 0; v < 4; ++v) {
+        sFt[le][v][pt] = dot2(mt[0], f[v], mt[1], g[v]);
+        sGt[le][v][pt] = dot2(mt[2], f[v], mt[3], g[v]);
+      }
     }
   }
   __syncthreads();
@@ -128,17 +122,17 @@ __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
       for (int v = 0; v < 4; ++v) Qo[v] = dw_from_double(qo[v]);
       const dw rhoo = (Qo[0] + k.p_ref) * rcp(Qo[3]);
       qc[0] = rho - rhoo;
-      qc[1] = rho * Q[1] - rhoo * Qo[1];
-      qc[2] = rho * Q[2] - rhoo * Qo[2];
-      qc[3] = (Q[0] - Qo[0]) * k.inv_gm1 +
-              half(rho * (Q[1] * Q[1] + Q[2] * Q[2]) - rhoo * (Qo[1] * Qo[1] + Qo[2] * Qo[2]));
+      qc[1] = dot2(rho, Q[1], -rhoo, Qo[1]);
+      qc[2] = dot2(rho, Q[2], -rhoo, Qo[2]);
+      qc[3] = mul_add(Q[0] - Qo[0], k.inv_gm1,
+                      half(dot2(rho, dot2(Q[1], Q[1], Q[2], Q[2]), -rhoo, dot2(Qo[1], Qo[1], Qo[2], Qo[2]))));
     } else {
       qc[0] = rho;
       qc[1] = rho * Q[1];
       qc[2] = rho * Q[2];
       qc[3] = rho * (Q[3] * k.inv_gm1 + half(Q[1] * Q[1] + Q[2] * Q[2]));
     }
-    const dw invJ = dw_from_double(mt[4]);
+    const dw ninvJ = -mt[4];
     const dw nodt = dw_from_double(-inv_odt);
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
@@ -160,12 +154,9 @@ __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
       acc.add_prod(sgL[j], com[0]);
       acc.add_prod(sgR[j], com[2]);
       // F = -acc / |J| - qc / (omega dt) + src - S
-      dw_acc F;
-      F.add_prod(-acc.value(), invJ);
-      F.add_prod(qc[v], nodt);
-      F.add(dw_from_double(Sv[v]));
+      const dw F = dot2_add(acc.value(), ninvJ, qc[v], nodt, dw_from_double(Sv[v]));
       const int row = v * N + pt;
-      sr[le][row] = scaled_in_dw<W>(F.value(), okS ? srs[le * n + row] : rs[(size_t)e * n + row]);
+      sr[le][row] = scaled_in_dw<W>(F, okS ? srs[le * n + row] : rs[(size_t)e * n + row]);
     }
   }
   __syncthreads();
@@ -214,7 +205,7 @@ static void dw_dispatch(const Ctx& c, const LevelDev& L, double* q, double inv_o
   const W* Dinv = (const W*)L.Dinv;
 #define PMG_VDW(PP)                                                                                         \
   volume_apply_dw_kernel<PP, W><<<blocks, threads, VolPrefetch<PP, W>::smem, s>>>(                          \
-      c.E, q, L.met, reinterpret_cast<const dw*>(L.Fcom), L.opw, c.phw, inv_odt, src, S, qref, Dinv, L.rs, L.cs, c.d_scal + 1)
+      c.E, q, L.metW, reinterpret_cast<const dw*>(L.Fcom), L.opw, c.phw, inv_odt, src, S, qref, Dinv, L.rs, L.cs, c.d_scal + 1)
   switch (L.P) {
     case 0: PMG_VDW(0); break;
     case 1: PMG_VDW(1); break;

@@ -46,132 +46,132 @@ inline PhysW make_physw(const Phys& ph) {
 __device__ __forceinline__ dw half(dw x) { return scale2(x, 0.5f); }
 __device__ __forceinline__ dw one_minus(dw x) { return dw{1.0f, 0.0f} - x; }
 
-// Convective part of flux_n of physics.cuh: (rho u_n, rho u_n u, rho u_n v,
-// rho u_n H); the pressure term pm n of the momentum rows is left to the
-// caller.
-__device__ __forceinline__ void flux_n_dw(const dw q[4], dw nx, dw ny, const PhysW& k, dw f[4]) {
-  const dw rho = q[0] * rcp(q[3]);
-  const dw H = k.Cp * q[3] + half(q[1] * q[1] + q[2] * q[2]);
-  const dw mn = rho * (q[1] * nx + q[2] * ny);
-  f[0] = mn;
-  f[1] = mn * q[1];
-  f[2] = mn * q[2];
-  f[3] = mn * H;
-}
-
 // roe_flux_jump of physics.cuh in double-word, without the pressure part
 // (pm^- + pm^+)/2 n dS of the central momentum flux: qm, qp hold absolute
 // pressure, dq = qp - qm (formed by the caller), (nx, ny) is the unit normal
 // and dS the face area.  The pressure part is the one large term of the
 // momentum rows (p ~ 1/(gamma Ma^2) when the absolute pressure is stored);
-// the caller adds it in binary64.
+// the caller adds it.  The arrangement is roe_jump_d's (half the area in the
+// mass fluxes, one reciprocal for 1/T and 1/p) with sums of products
+// renormalised once: about 1100 FP32 operations, 1400 as separate products and
+// sums.  64 elements (one GB300, launches of one warp's latency): the fused
+// P = 0 sweep 7.6 -> 5.6 us, the P = 1 face and update launches 5.2 -> 4.7 and
+// 6.4 -> 5.5 us, with the geometry kept in double-word and the states formed
+// on the FP32 pipes.
 __device__ __forceinline__ void roe_flux_jump_dw(const dw qm[4], const dw qp[4], const dw dq[4], dw nx, dw ny,
                                                  dw dS, const PhysW& k, dw out[4]) {
-  dw fm[4], fp[4];
-  flux_n_dw(qm, nx, ny, k, fm);
-  flux_n_dw(qp, nx, ny, k, fp);
+  const dw h = half(dS);
+  const dw mm = (qm[0] * rcp(qm[3])) * (dot2(qm[1], nx, qm[2], ny) * h);
+  const dw mp = (qp[0] * rcp(qp[3])) * (dot2(qp[1], nx, qp[2], ny) * h);
+  const dw Hm = mul_add(k.Cp, qm[3], half(dot2(qm[1], qm[1], qm[2], qm[2])));
+  const dw Hp = mul_add(k.Cp, qp[3], half(dot2(qp[1], qp[1], qp[2], qp[2])));
+  const dw f[4] = {mm + mp, dot2(mm, qm[1], mp, qp[1]), dot2(mm, qm[2], mp, qp[2]), dot2(mm, Hm, mp, Hp)};
   const dw dp = dq[0], du = dq[1], dv = dq[2], dT = dq[3];
   const dw p = qm[0] + half(dp);
   const dw u = qm[1] + half(du);
   const dw v = qm[2] + half(dv);
   const dw T = qm[3] + half(dT);
-  const dw iT = rcp(T);
-  const dw rho = p * iT;
-  const dw irho = T * rcp(p);
-  const dw c2 = k.gamma * T;
-  const dw vv = u * u + v * v;
-  const dw e2 = min_dw(dw{1.0f, 0.0f}, max_dw(k.eps_min2, vv * iT * k.inv_gamma));
+  const dw r = rcp(p * T);
+  const dw iT = p * r, irho = T * (T * r), rho = p * iT;
+  const dw c2 = k.gamma * T, ic2 = iT * k.inv_gamma;
+  const dw vv = dot2(u, u, v, v);
+  const dw e2 = min_dw(dw{1.0f, 0.0f}, max_dw(k.eps_min2, vv * ic2));
   const dw Ur2 = e2 * c2;
-  const dw ie2 = rcp(e2);
-  const dw iUr2 = ie2 * iT * k.inv_gamma;
-  const dw un = u * nx + v * ny;
-  const dw dun = du * nx + dv * ny;
-  const dw dut = dv * nx - du * ny;
-  const dw ome2 = one_minus(e2);
-  const dw alpha = half(ome2);
-  const dw aun2 = alpha * un;
-  const dw cpr = sqrt_dw(aun2 * aun2 + Ur2);
-  const dw unp = un - aun2;
-  const dw lp = unp + cpr, lm = unp - cpr;
-  const dw alp = abs_dw(lp), alm = abs_dw(lm), aun = abs_dw(un);
-  const dw a1 = (alp - alm) * half(rcp(cpr));
-  const dw a0 = alp - a1 * lp;
-  const dw rc2 = rho * c2;
-  const dw dpr = dp * irho;
+  const dw ie2 = rcp(e2), iUr2 = ie2 * ic2;
+  const dw un = dot2(u, nx, v, ny);
+  const dw dun = dot2(du, nx, dv, ny);
+  const dw bun = one_minus(e2) * un, hun = half(bun);
+  const dw cpr = sqrt_dw(mul_add(hun, hun, Ur2));
+  const dw uc = un - hun;
+  const dw lp = uc + cpr, lm = uc - cpr;
+  const dw alp = abs_dw(lp), aun = abs_dw(un);
+  const dw a1 = (alp - abs_dw(lm)) * half(rcp(cpr));
+  const dw a0 = mul_add(-a1, lp, alp);
+  const dw rc2 = rho * c2, dpr = dp * irho, a1e = a1 * e2;
   // |B| (dp, dun)
-  const dw zp = a0 * dp + a1 * (e2 * (un * dp + rc2 * dun));
-  const dw zu = a0 * dun + a1 * (dpr + un * dun);
-  // w = (B - u_n)^-1 (dp, dun)
-  const dw w0 = rho * dun;
-  const dw w1 = (dpr + ome2 * un * dun) * iUr2;
-  // (|B| - |u_n|) w
+  const dw zp = dot2(a0, dp, a1e, dot2(un, dp, rc2, dun));
+  const dw zu = dot2(a0, dun, a1, mul_add(un, dun, dpr));
+  // w = (B - u_n)^-1 (dp, dun), y = (|B| - |u_n|) w
+  const dw w0 = rho * dun, w1 = mul_add(bun, dun, dpr) * iUr2;
   const dw a0u = a0 - aun;
-  const dw y0 = a0u * w0 + a1 * (e2 * (un * w0 + rc2 * w1));
-  const dw y1 = a0u * w1 + a1 * (dun + un * w1);
+  const dw y0 = dot2(a0u, w0, a1e, dot2(un, w0, rc2, w1));
+  const dw y1 = dot2(a0u, w1, a1, mul_add(un, w1, dun));
   const dw irCp = irho * k.inv_Cp;
-  const dw xT = aun * dT + e2 * k.gm1 * T * y1 - ome2 * un * irCp * y0;
-  const dw xt = aun * dut;
-  const dw xu = zu * nx - xt * ny;
-  const dw xv = zu * ny + xt * nx;
+  const dw xT = dot3(aun, dT, Ur2 * k.inv_Cp, y1, -(bun * irCp), y0);
   // K then M
   const dw yp = zp * ie2;
-  const dw yT = (ie2 - dw{1.0f, 0.0f}) * irCp * zp + xT;
-  const dw drho = (yp - rho * yT) * iT;
-  const dw H = k.Cp * T + half(vv);
-  const dw d1 = u * drho + rho * xu;
-  const dw d2 = v * drho + rho * xv;
-  const dw d3 = H * drho - yp + rho * (u * xu + v * xv) + rho * k.Cp * yT;
-  const dw hdS = half(dS);
-  out[0] = ((fm[0] + fp[0]) - drho) * hdS;
-  out[1] = ((fm[1] + fp[1]) - d1) * hdS;
-  out[2] = ((fm[2] + fp[2]) - d2) * hdS;
-  out[3] = ((fm[3] + fp[3]) - d3) * hdS;
+  const dw yT = mul_add(irCp, yp - zp, xT);
+  const dw drho = mul_add(-rho, yT, yp) * iT;
+  const dw zz = mul_add(-aun, dun, zu);
+  const dw xu = dot2(aun, du, zz, nx), xv = dot2(aun, dv, zz, ny);
+  const dw H = mul_add(k.Cp, T, half(vv));
+  const dw vx = dot3(u, xu, v, xv, k.Cp, yT);
+  out[0] = mul_add(-h, drho, f[0]);
+  out[1] = mul_add(-h, dot2(u, drho, rho, xu), f[1]);
+  out[2] = mul_add(-h, dot2(v, drho, rho, xv), f[2]);
+  out[3] = mul_add(-h, dot2_add(H, drho, rho, vx, -yp), f[3]);
+}
+
+// States of one face point in double-word from its binary64 parts: the own
+// trace sm and the jump dq, both relative to the reference state (ref: p and T;
+// the velocity's reference is zero).  The sums run on the FP32 pipes: an FP64
+// instruction takes as long as 16 of theirs.  pg receives the gauge pressures'
+// sum p^- + p^+.
+__device__ __forceinline__ void face_states_dw(double ref_p, double ref_T, const double sm[4], const double dq[4],
+                                               const PhysW& k, dw Qm[4], dw Qp[4], dw DQ[4], dw& pg) {
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    Qm[v] = dw_from_double(sm[v]);
+    DQ[v] = dw_from_double(dq[v]);
+  }
+  const dw P = dw_from_double(ref_p) + Qm[0];
+  Qm[3] = dw_from_double(ref_T) + Qm[3];
+  pg = scale2(P, 2.0f) + DQ[0];
+  Qm[0] = P + k.p_ref;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) Qp[v] = Qm[v] + DQ[v];
 }
 
 // Common Roe flux of one face point from binary64 traces; DWF selects the
 // double-word evaluation (above; the central pressure term in binary64)
-// over the binary64 one.
+// over the binary64 one.  ref, sm, dq as in face_states_dw; sp = sm + dq.
 template <bool DWF>
-__device__ __forceinline__ void face_roe(const double qm[4], const double qp[4], const double dq[4], double pgm,
-                                         double pgp, double nx, double ny, double dS, const Phys& ph,
+__device__ __forceinline__ void face_roe(const double ref[4], const double sm[4], const double sp[4],
+                                         const double dq[4], double nx, double ny, double dS, const Phys& ph,
                                          const PhysW& phw, double out[4]) {
   if (DWF) {
-    dw Qm[4], Qp[4], DQ[4], o[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      Qm[v] = dw_from_double(qm[v]);
-      Qp[v] = dw_from_double(qp[v]);
-      DQ[v] = dw_from_double(dq[v]);
-    }
+    dw Qm[4], Qp[4], DQ[4], o[4], pg;
+    face_states_dw(ref[0], ref[3], sm, dq, phw, Qm, Qp, DQ, pg);
     roe_flux_jump_dw(Qm, Qp, DQ, dw_from_double(nx), dw_from_double(ny), dw_from_double(dS), phw, o);
-    const double pc = (pgm + pgp) * (0.5 * dS);
+    const double pc = ((ref[0] + sm[0]) + (ref[0] + sp[0])) * (0.5 * dS);
     out[0] = dw_to_double(o[0]);
     out[1] = fma(pc, nx, dw_to_double(o[1]));
     out[2] = fma(pc, ny, dw_to_double(o[2]));
     out[3] = dw_to_double(o[3]);
   } else {
-    const double n[2] = {nx, ny};
+    double qm[4], qp[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      qm[v] = ref[v] + sm[v];
+      qp[v] = ref[v] + sp[v];
+    }
+    const double pgm = qm[0], pgp = qp[0], n[2] = {nx, ny};   // gauge pressures for the momentum fluxes
+    qm[0] += ph.p_ref;   // absolute pressure for the averaged state and rho
+    qp[0] += ph.p_ref;
     roe_jump_d<2>(qm, qp, dq, pgm, pgp, n, dS, ph, out);
   }
 }
 // The double-word face flux left in double-word, the central pressure term
-// included: for gauge storage, where the momentum-flux pressures pgm, pgp
-// are the small p - p_ref.
-__device__ __forceinline__ void face_roe_dw(const double qm[4], const double qp[4], const double dq[4], double pgm,
-                                            double pgp, double nx, double ny, double dS, const PhysW& phw,
-                                            dw out[4]) {
-  dw Qm[4], Qp[4], DQ[4];
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    Qm[v] = dw_from_double(qm[v]);
-    Qp[v] = dw_from_double(qp[v]);
-    DQ[v] = dw_from_double(dq[v]);
-  }
-  const dw NX = dw_from_double(nx), NY = dw_from_double(ny), DS = dw_from_double(dS);
-  roe_flux_jump_dw(Qm, Qp, DQ, NX, NY, DS, phw, out);
-  const dw pc = half((dw_from_double(pgm) + dw_from_double(pgp)) * DS);
-  out[1] = out[1] + pc * NX;
-  out[2] = out[2] + pc * NY;
+// included: for gauge storage, where the momentum-flux pressures are the small
+// p - p_ref.  (nx, ny, dS): the double-word face geometry.
+__device__ __forceinline__ void face_roe_dw(double ref_p, double ref_T, const double sm[4], const double dq[4], dw nx,
+                                            dw ny, dw dS, const PhysW& phw, dw out[4]) {
+  dw Qm[4], Qp[4], DQ[4], pg;
+  face_states_dw(ref_p, ref_T, sm, dq, phw, Qm, Qp, DQ, pg);
+  roe_flux_jump_dw(Qm, Qp, DQ, nx, ny, dS, phw, out);
+  const dw pc = half(pg * dS);
+  out[1] = mul_add(pc, nx, out[1]);
+  out[2] = mul_add(pc, ny, out[2]);
 }
 #endif  // __CUDACC__
 

@@ -122,6 +122,8 @@ struct LevelDev {
   double* Pd = nullptr;        // restricted defect (coarse levels)
   double* met = nullptr;       // 5 * E * N (2D), 10 * E * N (3D)
   double* face = nullptr;      // E * 4 * n1 * 3 (2D), E * 6 * NF * 4 (3D)
+  dw* metW = nullptr;          // the same in double-word, for the sweeps (2D)
+  dw* faceW = nullptr;
   double* Fcom = nullptr;      // nv * E * faces * NF common fluxes, outward
   // viscous terms (mu > 0 only); hexahedra in brackets
   double* Gb = nullptr;        // 6 [12] * E * N broken gradients of (u, v, T) [(u, v, w, T)]:
