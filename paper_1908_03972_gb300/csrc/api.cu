@@ -386,7 +386,8 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
   PMG_CK(dalloc(&c.d_faces, fbuf.size()));
   PMG_CK(cudaMemcpy(c.d_faces, fbuf.data(), sizeof(int) * fbuf.size(), cudaMemcpyHostToDevice));
   size_t maxtot = 0;
-  int maxblocks = 1;
+  int maxblocks = 1, n_sms = 0;
+  PMG_CK(cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, c.device));
   size_t wbytes = c.cfg.block_prec == PMG_PREC_FP64 ? 8 : c.cfg.block_prec == PMG_PREC_BF16R ? 2 : 4;
   for (int l = 0; l < c.cfg.n_levels; ++l) {
     LevelDev& L = c.lev[l];
@@ -433,16 +434,27 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
         dalloc(&L.Fcom, (size_t)c.nv * c.E * c.nfc * L.NF) || dalloc(&L.Dfull, nn2) ||
         cudaMalloc(&L.Dinv, nn2 * wbytes) || dalloc(&L.rs, (size_t)c.E * L.n) || dalloc(&L.cs, (size_t)c.E * L.n))
       return fail(PMG_ENOMEM, "device allocation failed for level data");
-    // Coarse levels up to P = PMG_FUSE_MAX_P (default 0) are smoothed by the
-    // fused one-launch sweep (k_fused.cu), which evaluates every face from both
-    // of its elements.  At P = 0 the extra face work runs on SMSPs the split
-    // launches leave idle and the sweep saves a launch (C2 V-cycle 2.6%
-    // faster); from P = 1 on, the doubled face work costs more than it saves.
-    int fuse_max = 0;
-    if (const char* env = getenv("PMG_FUSE_MAX_P")) fuse_max = atoi(env);
+    // Small coarse levels are smoothed by a fused one-launch sweep (k_fused.cu,
+    // k3_fused.cu), which evaluates every face from both of its elements: the
+    // extra face work runs on SM sub-partitions the split launches leave idle and
+    // a launch is saved, until that work fills them.  The limits in elements per
+    // SM are where the two cross on 152 SMs: ten P{3-2-1-0} V-cycles with P = 0,
+    // P <= 1 and P <= 2 fused take, in double-word, 12.6 / 11.7 / 11.2 ms at 1024
+    // elements, 13.3 / 12.4 / 12.3 at 2304, 15.5 / 14.6 / 15.5 at 4096, 18.0 /
+    // 17.8 / 18.7 at 5184 and 20.0 / 20.0 / 21.2 at 6400; in binary64 21.0 /
+    // 20.3 / 20.0 at 1024, 24.4 / 24.1 / 25.9 at 2304 and 27.6 / 29.4 / 36.5 at
+    // 3136.  PMG_FUSE_MAX_P sets the highest fused P instead (-1: none).
     bool boundary = false;
     for (const FaceRec& fr : c.mesh.faces) boundary = boundary || fr.eR < 0;
-    L.fused = (c.dim == 2 && l > 0 && L.P <= fuse_max && L.P <= 3 && c.ph.mu == 0.0 && !boundary);
+    const bool words = flux_dw_sweep(c) && c.ph.p_ref != 0.0;
+    const int per_sm[3] = {1 << 20, words ? 36 : 16, words ? 16 : 8};
+    bool fuse = L.P <= 2 && c.E <= (long long)per_sm[L.P <= 2 ? L.P : 2] * n_sms;
+    bool fuse3 = fused3_applies(L.P, c.E, n_sms);
+    if (const char* env = getenv("PMG_FUSE_MAX_P")) {
+      fuse = L.P <= atoi(env) && L.P <= 3;
+      fuse3 = fuse3 && atoi(env) >= 0;
+    }
+    L.fused = l > 0 && (c.dim == 3 ? fuse3 : fuse && c.ph.mu == 0.0 && !boundary);
     // Coarse levels with P <= 1 that the double-word sweep arithmetic serves
     // (gauge storage, mu = 0, no boundary faces) may be smoothed by the fused
     // one-sweep kernel or by the multi-sweep tiles (k_tile.cu); pmg_autotune

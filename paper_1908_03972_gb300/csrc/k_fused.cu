@@ -469,6 +469,7 @@ static void fused_launch(const Ctx& c, const LevelDev& L, const double* qin, dou
 
 void launch_fused_sweep(const Ctx& c, const LevelDev& L, const double* qin, double* qout, double inv_odt,
                         const double* src, const double* S, const double* qref, int prec, cudaStream_t s) {
+  if (c.dim == 3) { launch_fused_sweep3(c, L, qin, qout, inv_odt, S, qref, prec, s); return; }
   switch (L.P) {
     case 0: fused_launch<0>(c, L, qin, qout, inv_odt, src, S, qref, prec, s); break;
     case 1: fused_launch<1>(c, L, qin, qout, inv_odt, src, S, qref, prec, s); break;

@@ -322,6 +322,10 @@ void launch_prolong3(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const
                      const double* qcb, double* qf, int add, cudaStream_t s);
 void launch_bsum_update3(const Ctx& c, int N, const double* qn, double* const* R, const double* b, int nr,
                          double dt, double* q, cudaStream_t s);
+// One-launch sweep of a small P = 0 level of hexahedra (k3_fused.cu).
+bool fused3_applies(int P, int E, int sms);
+void launch_fused_sweep3(const Ctx& c, const LevelDev& L, const double* qin, double* qout, double inv_odt,
+                         const double* S, const double* qref, int prec, cudaStream_t s);
 // Vector kernels of the Newton-Krylov solver (k_krylov.cu).
 constexpr int kDotBlocks = 304;
 struct Scale5 {
