@@ -724,8 +724,7 @@ static void vcycle_level(Ctx& c, int l, bool refresh) {
   const XferTab& X = c.xfer[l];
   {
     ProfScope ps(c, K_RESTRICT, l + 1);
-    launch_restrict(c, L, C, X, L.q, C.q, C.qb, 1.0, c.stream);       // q^b = P q^a
-    launch_restrict(c, L, C, X, L.F, C.Pd, nullptr, -1.0, c.stream);  // P d = -P (F - S)
+    launch_restrict_fas(c, L, C, X, L.q, C.q, C.qb, L.F, C.Pd, c.stream);   // q^b = P q^a, P d = -P (F - S)
   }
   {
     ProfScope ps(c, K_FACE, l + 1);
@@ -1702,7 +1701,7 @@ pmg_status pmg_restrict(pmg_ctx* h, int lf, const double* qf, double* qc, int on
     in = c.d_tmp0;
     out = c.d_tmp1;
   }
-  launch_restrict(c, F, C, c.xfer[lf], in, out, nullptr, 1.0, c.stream);
+  launch_restrict(c, F, C, c.xfer[lf], in, out, c.stream);
   PMG_CK_LAUNCH();
   if (!on_device) PMG_CK(copy_out(c, qc, out, C.tot, 0));
   else PMG_CK(cudaStreamSynchronize(c.stream));

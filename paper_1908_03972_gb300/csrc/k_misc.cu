@@ -4,102 +4,6 @@
 
 namespace pmg {
 
-// Restriction: out[v][e][(jc,ic)] = sum_{a,b} R[ic][a] R[jc][b] in[v][e][(b,a)]
-// (tensor product of the 1D L2 projection).  Optionally also writes a copy
-// (out2) and scales the result (scale = -1 turns F - S into the defect).
-template <int PF, int PC>
-__global__ void restrict_kernel(int E, XferTab X, const double* __restrict__ in, double* __restrict__ out,
-                                double* __restrict__ out2, double scale) {
-  constexpr int nf = PF + 1, nc = PC + 1, Nf = nf * nf, Nc = nc * nc;
-  __shared__ double sR[nc][nf];
-  if (threadIdx.x < nc * nf) sR[threadIdx.x / nf][threadIdx.x % nf] = X.R[threadIdx.x / nf][threadIdx.x % nf];
-  __syncthreads();
-  int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= E * Nc) return;
-  int e = tid / Nc, cp = tid - e * Nc, ic = cp % nc, jc = cp / nc;
-  for (int v = 0; v < 4; ++v) {
-    const double* src = in + ((size_t)v * E + e) * Nf;
-    double s = 0.0;
-#pragma unroll
-    for (int b = 0; b < nf; ++b) {
-      double t = 0.0;
-#pragma unroll
-      for (int a = 0; a < nf; ++a) t = fma(sR[ic][a], src[b * nf + a], t);
-      s = fma(sR[jc][b], t, s);
-    }
-    s *= scale;
-    size_t o = ((size_t)v * E + e) * Nc + cp;
-    out[o] = s;
-    if (out2) out2[o] = s;
-  }
-}
-
-// Prolongation of the coarse correction: qf += I (qc - qcb), or qf = I qc
-// when qcb is null and add = 0.
-template <int PF, int PC>
-__global__ void prolong_kernel(int E, XferTab X, const double* __restrict__ qc, const double* __restrict__ qcb,
-                               double* __restrict__ qf, int add) {
-  constexpr int nf = PF + 1, nc = PC + 1, Nf = nf * nf, Nc = nc * nc;
-  __shared__ double sI[nf][nc];
-  if (threadIdx.x < nf * nc) sI[threadIdx.x / nc][threadIdx.x % nc] = X.I[threadIdx.x / nc][threadIdx.x % nc];
-  __syncthreads();
-  int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= E * Nf) return;
-  int e = tid / Nf, fp = tid - e * Nf, i = fp % nf, j = fp / nf;
-  for (int v = 0; v < 4; ++v) {
-    const double* a0 = qc + ((size_t)v * E + e) * Nc;
-    const double* b0 = qcb ? qcb + ((size_t)v * E + e) * Nc : nullptr;
-    double s = 0.0;
-#pragma unroll
-    for (int b = 0; b < nc; ++b) {
-      double t = 0.0;
-#pragma unroll
-      for (int a = 0; a < nc; ++a) {
-        double c = a0[b * nc + a];
-        if (b0) c -= b0[b * nc + a];
-        t = fma(sI[i][a], c, t);
-      }
-      s = fma(sI[j][b], t, s);
-    }
-    size_t o = ((size_t)v * E + e) * Nf + fp;
-    if (add) qf[o] += s;
-    else qf[o] = s;
-  }
-}
-
-#define PMG_PAIRS(M) \
-  M(1, 0) M(2, 0) M(2, 1) M(3, 0) M(3, 1) M(3, 2) M(4, 0) M(4, 1) M(4, 2) M(4, 3) M(5, 0) M(5, 1) M(5, 2) M(5, 3) M(5, 4)
-
-void launch_restrict(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const XferTab& X, const double* in,
-                     double* out, double* out2, double scale, cudaStream_t s) {
-  if (c.dim == 3) { launch_restrict3(c, Lf, Lc, X, in, out, out2, scale, s); return; }
-  int total = c.E * Lc.N, threads = 64, blocks = (total + threads - 1) / threads;
-#define PMG_R(A, B) \
-  if (Lf.P == A && Lc.P == B) { restrict_kernel<A, B><<<blocks, threads, 0, s>>>(c.E, X, in, out, out2, scale); return; }
-  PMG_PAIRS(PMG_R)
-#undef PMG_R
-}
-
-static void prolong_impl(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const XferTab& X, const double* qc,
-                         const double* qcb, double* qf, int add, cudaStream_t s) {
-  if (c.dim == 3) { launch_prolong3(c, Lf, Lc, X, qc, qcb, qf, add, s); return; }
-  int total = c.E * Lf.N, threads = 64, blocks = (total + threads - 1) / threads;
-#define PMG_P(A, B) \
-  if (Lf.P == A && Lc.P == B) { prolong_kernel<A, B><<<blocks, threads, 0, s>>>(c.E, X, qc, qcb, qf, add); return; }
-  PMG_PAIRS(PMG_P)
-#undef PMG_P
-}
-
-void launch_prolong_add(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const XferTab& X, const double* qc,
-                        const double* qcb, double* qf, cudaStream_t s) {
-  prolong_impl(c, Lf, Lc, X, qc, qcb, qf, 1, s);
-}
-
-void launch_prolong(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const XferTab& X, const double* in,
-                    double* out, cudaStream_t s) {
-  prolong_impl(c, Lf, Lc, X, in, nullptr, out, 0, s);
-}
-
 // ------------------------------------------------------------------ stages
 __global__ void cons_kernel(size_t plane, Phys ph, const double* __restrict__ q, double* __restrict__ qc) {
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;

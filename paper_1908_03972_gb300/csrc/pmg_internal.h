@@ -285,7 +285,10 @@ void launch_factor(const Ctx& c, LevelDev& L, int level, int prec, int* flag, cu
 void launch_apply(const Ctx& c, const LevelDev& L, int prec, const double* r, double* x, int accumulate,
                   cudaStream_t s);
 void launch_restrict(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const XferTab& X, const double* in,
-                     double* out, double* out2, double scale, cudaStream_t s);
+                     double* out, cudaStream_t s);
+// The FAS restriction: qc = qcb = R q and Pd = -R F
+void launch_restrict_fas(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const XferTab& X, const double* q,
+                         double* qc, double* qcb, const double* F, double* Pd, cudaStream_t s);
 void launch_prolong_add(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const XferTab& X, const double* qc,
                         const double* qcb, double* qf, cudaStream_t s);
 void launch_prolong(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const XferTab& X, const double* in,
@@ -316,10 +319,6 @@ int residual_blocks_for3(int P, int E);
 void launch_grad3(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s);
 void launch_apply3(const Ctx& c, const LevelDev& L, int prec, const double* r, double* x, int accumulate,
                    cudaStream_t s);
-void launch_restrict3(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const XferTab& X, const double* in,
-                      double* out, double* out2, double scale, cudaStream_t s);
-void launch_prolong3(const Ctx& c, const LevelDev& Lf, const LevelDev& Lc, const XferTab& X, const double* qc,
-                     const double* qcb, double* qf, int add, cudaStream_t s);
 void launch_bsum_update3(const Ctx& c, int N, const double* qn, double* const* R, const double* b, int nr,
                          double dt, double* q, cudaStream_t s);
 // One-launch sweep of a small P = 0 level of hexahedra (k3_fused.cu).
