@@ -533,6 +533,8 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
   if (c.dim == 2) {
     PMG_CK(prepare_residual_kernels(c));
     PMG_CK(prepare_volume_dw_kernels(c));
+  } else {
+    PMG_CK(prepare_apply3(c));
   }
   if (c.ph.p_ref != 0.0 && c.mesh.Ng > 1)
     for (int l = 1; l < c.cfg.n_levels; ++l)

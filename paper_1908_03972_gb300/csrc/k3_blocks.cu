@@ -2,21 +2,105 @@
 // (Section 2.4, eq. smoothing_element_jacobi, d = 3): x = cs .* (D^-1 (rs .* r))
 // with the factored inverse (column-major); one thread per solution point forms
 // its point's five rows, so the threads of an element read every column
-// contiguously.  Bound by the stream of the inverses, so ten columns' loads are
-// in flight per thread.
+// contiguously.  Bound by the stream of the inverses (n^2 entries per element,
+// read once).  Loaded into registers inside the product loop, the columns in
+// flight are what a thread can hold (ten), which leaves HBM half idle at
+// n = 320; here KC columns of each element at a time go through a ring of S
+// stages in shared memory with 16-byte asynchronous copies.  The columns are
+// used in the order of the plain loop, so the sums are the same bit for bit.
+// Measured on one GB300, FP32, us (before, columns in registers): 960 elements of
+// n = 320 97.6 -> 68.4 (393 MB, 5.7 TB/s), of n = 135 37.1 -> 28.3; 2304 of
+// n = 135 42.9 -> 37.6, of n = 40 12.9 -> 8.2.  Inside the residual-and-update
+// kernel (k3_residual.cu) the ring takes the shared memory that its resident
+// CTAs need (n = 320: 104 -> 158 us), so that keeps its columns in registers.
 // Assembly and factorisation: k_assemble.cu, k_factor.cu.
 #include "pmg_internal.h"
 #include "physics3.cuh"
 
 namespace pmg {
 
+// One element's chunk of KC columns starts at any multiple of the entry size
+// when its columns are not multiples of 16 bytes (n = 135): it is copied from
+// the 16-byte boundary at or below its first entry, and pieces that would pass
+// the array's end are read entry by entry.
+static __device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+static __device__ __forceinline__ void async_wait() {   // all but the N newest groups have landed
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+template <class W, int n, int EPB, int KC, int S>
+struct BlockStream {
+  static constexpr int colB = n * (int)sizeof(W), chunkB = KC * colB, NC = (n + KC - 1) / KC;
+  static constexpr bool aligned = chunkB % 16 == 0 && (n * colB) % 16 == 0;
+  static constexpr int segB = (chunkB + (aligned ? 0 : 15) + 15) / 16 * 16;   // one element's chunk
+  static constexpr int stageB = segB * EPB;
+  static constexpr size_t bytes = (size_t)S * stageB;
+
+  // Chunk c of the elements e0 .. e0 + ne - 1 into its stage (one group per
+  // call, empty past the last chunk).
+  static __device__ __forceinline__ void issue(unsigned char* ring, const W* __restrict__ Dinv, int E, int e0, int ne,
+                                               int c) {
+    if (c < NC) {
+      constexpr int pieces = segB / 16;
+      unsigned char* st = ring + (size_t)(c % S) * stageB;
+      const size_t total = (size_t)E * n * colB;
+      for (int t = threadIdx.x; t < ne * pieces; t += blockDim.x) {
+        const int le = t / pieces, p = t - le * pieces;
+        const size_t off = (size_t)(e0 + le) * n * colB + (size_t)c * chunkB;   // first byte of the chunk
+        const size_t src = (aligned ? off : off & ~(size_t)15) + 16 * (size_t)p;
+        const size_t end = off + (size_t)(c == NC - 1 ? (n - c * KC) * colB : chunkB);
+        unsigned char* dst = st + le * segB + 16 * p;
+        if (src >= end) continue;
+        if (aligned || src + 16 <= total) {
+          const unsigned int d = (unsigned int)__cvta_generic_to_shared(dst);
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d),
+                       "l"(reinterpret_cast<const unsigned char*>(Dinv) + src)
+                       : "memory");
+        } else {
+          for (size_t b = src; b < total; b += sizeof(W))
+            *reinterpret_cast<W*>(dst + (b - src)) = Dinv[b / sizeof(W)];
+        }
+      }
+    }
+    async_commit();
+  }
+  // Column 0 of chunk c of local element le.
+  static __device__ __forceinline__ const W* columns(const unsigned char* ring, int e0, int le, int c) {
+    const unsigned char* s = ring + (size_t)(c % S) * stageB + le * segB;
+    if (!aligned) s += ((size_t)(e0 + le) * n * colB + (size_t)c * chunkB) & 15;
+    return reinterpret_cast<const W*>(s);
+  }
+};
+
+// Elements per CTA (one or two warps), columns per chunk and stages.
+template <int P>
+struct ApplyEPB3 {
+  static constexpr int value = P == 0 ? 64 : P == 1 ? 8 : P == 2 ? 2 : 1;
+};
+constexpr int kStages3 = 4;
+template <int P>
+struct StreamCols3 {
+  static constexpr int value = P == 1 ? 5 : 4;
+};
+template <class W, int P>
+using Stream3 =
+    BlockStream<W, 5 * (P + 1) * (P + 1) * (P + 1), ApplyEPB3<P>::value, StreamCols3<P>::value, kStages3>;
+template <class W, int P>
+constexpr size_t stream3_bytes() { return P == 0 ? 0 : Stream3<W, P>::bytes; }
+
 template <class W, int P>
 __global__ void __launch_bounds__(64) apply3_kernel(int E, const W* __restrict__ Dinv, const double* __restrict__ rs,
                                                     const double* __restrict__ cs, const double* __restrict__ r,
                                                     double* __restrict__ x, int accumulate) {
   constexpr int N = (P + 1) * (P + 1) * (P + 1), n = 5 * N;
-  constexpr int EPB = N <= 32 ? 64 / N : 1;
+  constexpr int EPB = ApplyEPB3<P>::value;
   using Acc = typename Blk<W>::acc;
+  using Stream = Stream3<W, P>;
+  extern __shared__ __align__(16) unsigned char ring[];
+  const int e0 = blockIdx.x * EPB, ne = min(EPB, E - e0);
+  if (P > 0)
+    for (int c = 0; c < kStages3 - 1; ++c) Stream::issue(ring, Dinv, E, e0, ne, c);
   __shared__ Acc sr[EPB][n];
   const int le = threadIdx.x / N, pt = threadIdx.x - le * N;
   const int e = blockIdx.x * EPB + le;
@@ -27,15 +111,38 @@ __global__ void __launch_bounds__(64) apply3_kernel(int E, const W* __restrict__
     for (int v = 0; v < 5; ++v)
       sr[le][v * N + pt] = scaled_in<W>(r[v * plane + (size_t)e * N + pt], rs[(size_t)e * n + v * N + pt]);
   }
-  __syncthreads();
-  if (!active) return;
   Acc acc[5] = {0, 0, 0, 0, 0};
-  const W* Dm = Dinv + (size_t)e * n * n + pt;
-#pragma unroll 10
-  for (int k = 0; k < n; ++k) {
-    const Acc rk = sr[le][k];
+  if (P > 0) {
+#pragma unroll 1
+    for (int c = 0; c < Stream::NC; ++c) {
+      async_wait<kStages3 - 2>();
+      __syncthreads();   // chunk c (and, the first time, sr) visible; the stage of chunk c - 1 free
+      Stream::issue(ring, Dinv, E, e0, ne, c + kStages3 - 1);
+      if (active) {
+        const W* Dm = Stream::columns(ring, e0, le, c) + pt;
+        const Acc* rk = sr[le] + c * StreamCols3<P>::value;
+        const int nk = min(StreamCols3<P>::value, n - c * StreamCols3<P>::value);
 #pragma unroll
-    for (int v = 0; v < 5; ++v) acc[v] = fma(blk_val(__ldg(Dm + (size_t)k * n + v * N)), rk, acc[v]);
+        for (int kk = 0; kk < StreamCols3<P>::value; ++kk) {
+          if (kk < nk) {
+            const Acc rr = rk[kk];
+#pragma unroll
+            for (int v = 0; v < 5; ++v) acc[v] = fma(blk_val(Dm[kk * n + v * N]), rr, acc[v]);
+          }
+        }
+      }
+    }
+    if (!active) return;
+  } else {
+    __syncthreads();
+    if (!active) return;
+    const W* Dm = Dinv + (size_t)e * n * n + pt;
+#pragma unroll
+    for (int k = 0; k < (P == 0 ? n : 0); ++k) {
+      const Acc rr = sr[le][k];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) acc[v] = fma(blk_val(__ldg(Dm + (size_t)k * n + v * N)), rr, acc[v]);
+    }
   }
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
@@ -50,9 +157,9 @@ template <class W>
 static void apply3_dispatch(const Ctx& c, const LevelDev& L, const double* r, double* x, int acc, cudaStream_t s) {
   const W* Dinv = (const W*)L.Dinv;
   const int N = L.N;
-  const int epb = N <= 32 ? 64 / N : 1;
+  const int epb = N == 1 ? ApplyEPB3<0>::value : N == 8 ? ApplyEPB3<1>::value : N == 27 ? ApplyEPB3<2>::value : ApplyEPB3<3>::value;
   const int threads = (epb * N + 31) / 32 * 32, blocks = (c.E + epb - 1) / epb;
-#define PMG_AP3(PP) apply3_kernel<W, PP><<<blocks, threads, 0, s>>>(c.E, Dinv, L.rs, L.cs, r, x, acc)
+#define PMG_AP3(PP) apply3_kernel<W, PP><<<blocks, threads, stream3_bytes<W, PP>(), s>>>(c.E, Dinv, L.rs, L.cs, r, x, acc)
   switch (L.P) {
     case 0: PMG_AP3(0); break;
     case 1: PMG_AP3(1); break;
@@ -60,6 +167,28 @@ static void apply3_dispatch(const Ctx& c, const LevelDev& L, const double* r, do
     default: PMG_AP3(3); break;
   }
 #undef PMG_AP3
+}
+
+// Ring of the apply kernels beyond the default shared memory.
+template <class W>
+static cudaError_t prepare3(int P) {
+  constexpr cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  switch (P) {
+    case 0: return cudaSuccess;
+    case 1: return cudaFuncSetAttribute(apply3_kernel<W, 1>, a, (int)stream3_bytes<W, 1>());
+    case 2: return cudaFuncSetAttribute(apply3_kernel<W, 2>, a, (int)stream3_bytes<W, 2>());
+    default: return cudaFuncSetAttribute(apply3_kernel<W, 3>, a, (int)stream3_bytes<W, 3>());
+  }
+}
+cudaError_t prepare_apply3(const Ctx& c) {
+  for (int l = 0; l < c.cfg.n_levels; ++l) {
+    const int P = c.lev[l].P;
+    const cudaError_t e = c.cfg.block_prec == PMG_PREC_FP64    ? prepare3<double>(P)
+                          : c.cfg.block_prec == PMG_PREC_BF16R ? prepare3<__nv_bfloat16>(P)
+                                                               : prepare3<float>(P);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 void launch_apply3(const Ctx& c, const LevelDev& L, int prec, const double* r, double* x, int accumulate,

@@ -317,6 +317,7 @@ void launch_volume_apply3(const Ctx& c, const LevelDev& L, double* q, double inv
 int residual_blocks_for3(int P, int E);
 // broken gradients of the viscous terms on hexahedra (Gb, 12 planes)
 void launch_grad3(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s);
+cudaError_t prepare_apply3(const Ctx& c);
 void launch_apply3(const Ctx& c, const LevelDev& L, int prec, const double* r, double* x, int accumulate,
                    cudaStream_t s);
 void launch_bsum_update3(const Ctx& c, int N, const double* qn, double* const* R, const double* b, int nr,
