@@ -8,11 +8,17 @@ namespace pmg {
 // Elements per CTA of the volume kernels.  Their threads are bound by FP64
 // issue (binary64: 2 DFMA per clock per SM) or by the latency of their chain
 // (double-word), so small CTAs of one or two warps spread even the coarse
-// levels (4096 elements) over all 152 SMs.
+// levels (4096 elements) over all 152 SMs.  An FP64 instruction takes its
+// 64 cycles whatever the active lanes, so the points should fill their warps:
+// at P = 4 five elements (125 of 128 lanes; two filled 50 of 64) take the
+// residual of 16384 viscous elements from 136 to 110 us and the BF16 update
+// from 231 to 204, although the five inverses no longer fit the prefetch; at
+// P = 5 three (108 of 128; one filled 36 of 64) take 1073 elements from 16.2
+// to 12.5 us.
 template <int P>
 struct ElemsPerBlock {
   static constexpr int N = (P + 1) * (P + 1);
-  static constexpr int value = P == 0 ? 32 : P == 1 ? 8 : P == 2 ? 7 : P == 3 ? 4 : P == 4 ? 2 : 1;
+  static constexpr int value = P == 0 ? 32 : P == 1 ? 8 : P == 2 ? 7 : P == 3 ? 4 : P == 4 ? 5 : 3;
 };
 
 // Prefetch layout of the residual-and-update sweep: the CTA's common face
