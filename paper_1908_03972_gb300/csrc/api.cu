@@ -567,6 +567,28 @@ static cudaError_t copy_out(const Ctx& c, double* dst, const double* src, size_t
   return cudaStreamSynchronize(c.stream);
 }
 
+// Whether this context's kernels may read or write p themselves: memory of its
+// own device (a copy takes peers' memory too, a kernel only what is mapped).
+static bool own_memory(const Ctx& c, const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == c.device;
+}
+
+// A caller's state into dst as the device holds it (pressure relative to p_gauge).
+static cudaError_t state_in(const Ctx& c, double* dst, const double* src, const LevelDev& L, int on_device) {
+  if (on_device && own_memory(c, src)) {
+    launch_copy_shift(L.tot / c.nv, L.tot, -c.ph.p_ref, src, dst, c.stream);
+    return cudaGetLastError();
+  }
+  const cudaError_t e = copy_in(c, dst, src, L.tot, on_device);
+  if (e == cudaSuccess) launch_shift_pressure(L.tot / c.nv, -c.ph.p_ref, dst, c.stream);
+  return e;
+}
+
 static int residual_block_count(const Ctx& c, int l) {
   return c.dim == 3 ? residual_blocks_for3(c.lev[l].P, c.E) : residual_blocks_for(c.lev[l].P, c.E);
 }
@@ -1374,8 +1396,7 @@ pmg_status pmg_set_state(pmg_ctx* h, int level, const double* q, int on_device) 
   Ctx& c = h->c;
   pmg_status st = check_level(c, level);
   if (st) return st;
-  PMG_CK(copy_in(c, c.lev[level].q, q, c.lev[level].tot, on_device));
-  launch_shift_pressure(c.lev[level].tot / c.nv, -c.ph.p_ref, c.lev[level].q, c.stream);
+  PMG_CK(state_in(c, c.lev[level].q, q, c.lev[level], on_device));
   PMG_CK_LAUNCH();
   PMG_CK(cudaStreamSynchronize(c.stream));
   if (level == 0) c.F0_valid = false;
@@ -1491,10 +1512,11 @@ pmg_status pmg_get_state(pmg_ctx* h, int level, double* q, int on_device) {
   pmg_status st = check_level(c, level);
   if (st) return st;
   const LevelDev& L = c.lev[level];
-  PMG_CK(cudaMemcpyAsync(c.d_tmp0, L.q, L.tot * 8, cudaMemcpyDeviceToDevice, c.stream));
-  launch_shift_pressure(L.tot / c.nv, c.ph.p_ref, c.d_tmp0, c.stream);
+  const bool direct = on_device && own_memory(c, q);
+  launch_copy_shift(L.tot / c.nv, L.tot, c.ph.p_ref, L.q, direct ? q : c.d_tmp0, c.stream);
   PMG_CK_LAUNCH();
-  PMG_CK(copy_out(c, q, c.d_tmp0, L.tot, on_device));
+  if (!direct) PMG_CK(copy_out(c, q, c.d_tmp0, L.tot, on_device));
+  else PMG_CK(cudaStreamSynchronize(c.stream));
   return PMG_OK;
 }
 
@@ -1504,8 +1526,7 @@ pmg_status pmg_residual(pmg_ctx* h, int level, const double* q, double* R, int o
   pmg_status st = check_level(c, level);
   if (st) return st;
   LevelDev& L = c.lev[level];
-  PMG_CK(copy_in(c, c.d_tmp0, q, L.tot, on_device));
-  launch_shift_pressure(L.tot / c.nv, -c.ph.p_ref, c.d_tmp0, c.stream);
+  PMG_CK(state_in(c, c.d_tmp0, q, L, on_device));
   const double* qd = c.d_tmp0;
   double* Rd = on_device ? R : c.d_tmp1;
   launch_face_flux(c, L, qd, c.stream);
@@ -1564,8 +1585,7 @@ pmg_status pmg_residual_static(pmg_ctx* h, int level, const double* q, double* R
     L.Gb = scratch + n_state + n_face;
     L.Qj = L.Gb + n_grad;
   }
-  PMG_CK(cudaMemcpyAsync(qs, q, n_state * 8, cudaMemcpyDeviceToDevice, c.stream));
-  launch_shift_pressure(n_state / c.nv, -c.ph.p_ref, qs, c.stream);
+  PMG_CK(state_in(c, qs, q, L, 1));
   launch_face_flux(c, L, qs, c.stream);
   launch_volume(c, L, level, qs, R, RES_PURE, 0.0, nullptr, nullptr, nullptr, nullptr, nullptr, c.stream);
   add_gauge_constant(c, level, R);
@@ -1595,8 +1615,7 @@ pmg_status pmg_stage_residual(pmg_ctx* h, int level, const double* q, double* F,
   if (st) return st;
   if (!c.stage_ready) return fail(PMG_ESTATE, "stage data not set");
   LevelDev& L = c.lev[level];
-  PMG_CK(copy_in(c, c.d_tmp0, q, L.tot, on_device));
-  launch_shift_pressure(L.tot / c.nv, -c.ph.p_ref, c.d_tmp0, c.stream);
+  PMG_CK(state_in(c, c.d_tmp0, q, L, on_device));
   const double* qd = c.d_tmp0;
   double* Fd = on_device ? F : c.d_tmp1;
   launch_face_flux(c, L, qd, c.stream);

@@ -298,6 +298,7 @@ void launch_stage_src(const Ctx& c, int N, const double* qcn, double* const* R, 
                       double dt, double inv_odt, double* src, cudaStream_t s);
 void launch_bsum_update(const Ctx& c, int N, const double* qn, double* const* R, const double* b, int nr,
                         double dt, double* q, cudaStream_t s);
+void launch_copy_shift(size_t plane, size_t n, double delta, const double* in, double* out, cudaStream_t s);
 void launch_shift_pressure(size_t plane, double delta, double* q, cudaStream_t s);
 void launch_dtau_min(const Ctx& c, double* partial, double* out, cudaStream_t s);
 void launch_grad(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s);
