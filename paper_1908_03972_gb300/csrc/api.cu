@@ -434,8 +434,8 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
         dalloc(&L.Fcom, (size_t)c.nv * c.E * c.nfc * L.NF) || dalloc(&L.Dfull, nn2) ||
         cudaMalloc(&L.Dinv, nn2 * wbytes) || dalloc(&L.rs, (size_t)c.E * L.n) || dalloc(&L.cs, (size_t)c.E * L.n))
       return fail(PMG_ENOMEM, "device allocation failed for level data");
-    // Small coarse levels are smoothed by a fused one-launch sweep (k_fused.cu,
-    // k3_fused.cu), which evaluates every face from both of its elements: the
+    // Small levels are smoothed by a fused one-launch sweep (k_fused.cu; coarse
+    // P = 0 levels of hexahedra k3_fused.cu), which evaluates every face from both of its elements: the
     // extra face work runs on SM sub-partitions the split launches leave idle and
     // a launch is saved, until that work fills them.  The limits in elements per
     // SM are where the two cross on 152 SMs: ten P{3-2-1-0} V-cycles with P = 0,
@@ -443,7 +443,9 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
     // elements, 13.3 / 12.4 / 12.3 at 2304, 15.5 / 14.6 / 15.5 at 4096, 18.0 /
     // 17.8 / 18.7 at 5184 and 20.0 / 20.0 / 21.2 at 6400; in binary64 21.0 /
     // 20.3 / 20.0 at 1024, 24.4 / 24.1 / 25.9 at 2304 and 27.6 / 29.4 / 36.5 at
-    // 3136.  PMG_FUSE_MAX_P sets the highest fused P instead (-1: none).
+    // 3136; with a P = 2 finest level, fused against split, ten P{2-1-0}
+    // V-cycles take 4.71 / 4.88 ms at 64 and 5.36 / 5.50 at 1600 elements in
+    // double-word, 8.28 / 8.50 at 64 in binary64.  PMG_FUSE_MAX_P sets the highest fused P instead (-1: none).
     bool boundary = false;
     for (const FaceRec& fr : c.mesh.faces) boundary = boundary || fr.eR < 0;
     const bool words = flux_dw_sweep(c) && c.ph.p_ref != 0.0;
@@ -454,7 +456,7 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
       fuse = L.P <= atoi(env) && L.P <= 3;
       fuse3 = fuse3 && atoi(env) >= 0;
     }
-    L.fused = l > 0 && (c.dim == 3 ? fuse3 : fuse && c.ph.mu == 0.0 && !boundary);
+    L.fused = c.dim == 3 ? l > 0 && fuse3 : fuse && c.ph.mu == 0.0 && !boundary;
     // Coarse levels with P <= 1 that the double-word sweep arithmetic serves
     // (gauge storage, mu = 0, no boundary faces) may be smoothed by the fused
     // one-sweep kernel or by the multi-sweep tiles (k_tile.cu); pmg_autotune
@@ -667,7 +669,8 @@ static void refresh_level(Ctx& c, int l) {
 // on the level system).  With F_valid, lev[l].F already holds F_l(q) - S_l
 // for the current state and the first sweep only applies the blocks; every
 // other sweep is one face-flux launch and one volume launch that forms the
-// residual and updates the state in place.  final_residual leaves
+// residual and updates the state in place, or one fused launch (coarse
+// levels then form the first residual again).  final_residual leaves
 // F_l(q) - S_l of the smoothed state in lev[l].F (and its norm, if asked).
 // Fused levels return the number of state-buffer swaps.
 static int sweeps(Ctx& c, int l, int n, bool F_valid, bool final_residual, bool final_norm) {
@@ -686,23 +689,25 @@ static int sweeps(Ctx& c, int l, int n, bool F_valid, bool final_residual, bool 
     if (final_residual) system_residual(c, l, final_norm);
     return swaps;
   }
+  const double *qref = l > 0 ? L.qb : (c.split_stage ? c.qn : nullptr), *src = l == 0 ? c.src : nullptr,
+               *S = l > 0 ? L.S : nullptr;
+  int s = 0;
+  if (F_valid && n > 0 && (l == 0 || !L.fused)) {
+    ProfScope ps(c, K_APPLY, l);
+    launch_apply(c, L, c.cfg.block_prec, L.F, L.q, 1, c.stream);
+    s = 1;
+  }
   if (L.fused) {
-    for (int s = 0; s < n; ++s) {
+    const int swaps = n - s;
+    for (; s < n; ++s) {
       {
         ProfScope ps(c, K_FUSED, l);
-        launch_fused_sweep(c, L, L.q, L.q2, 1.0 / c.omega_dt, nullptr, L.S, L.qb, c.cfg.block_prec, c.stream);
+        launch_fused_sweep(c, L, L.q, L.q2, 1.0 / c.omega_dt, src, S, qref, c.cfg.block_prec, c.stream);
       }
       std::swap(L.q, L.q2);
     }
     if (final_residual) system_residual(c, l, final_norm);
-    return n;
-  }
-  const double* qref = l > 0 ? L.qb : (c.split_stage ? c.qn : nullptr);
-  int s = 0;
-  if (F_valid && n > 0) {
-    ProfScope ps(c, K_APPLY, l);
-    launch_apply(c, L, c.cfg.block_prec, L.F, L.q, 1, c.stream);
-    s = 1;
+    return swaps;
   }
   for (; s < n; ++s) {
     {
@@ -712,11 +717,9 @@ static int sweeps(Ctx& c, int l, int n, bool F_valid, bool final_residual, bool 
     {
       ProfScope ps(c, K_VOLUME, l);
       if (volume_dw_applies(c))
-        launch_volume_apply_dw(c, L, L.q, 1.0 / c.omega_dt, l == 0 ? c.src : nullptr, l > 0 ? L.S : nullptr, qref,
-                               c.cfg.block_prec, c.stream);
+        launch_volume_apply_dw(c, L, L.q, 1.0 / c.omega_dt, src, S, qref, c.cfg.block_prec, c.stream);
       else
-        launch_volume_apply(c, L, L.q, 1.0 / c.omega_dt, l == 0 ? c.src : nullptr, l > 0 ? L.S : nullptr, qref,
-                            c.cfg.block_prec, c.stream);
+        launch_volume_apply(c, L, L.q, 1.0 / c.omega_dt, src, S, qref, c.cfg.block_prec, c.stream);
     }
   }
   if (final_residual) system_residual(c, l, final_norm);

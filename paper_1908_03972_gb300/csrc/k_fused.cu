@@ -242,8 +242,9 @@ template <int P, class W>
 __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
     int E, const double* __restrict__ qin, double* __restrict__ qout, const dw* __restrict__ met,
     const dw* __restrict__ face, const int* __restrict__ nbr, OpTabW opw, OpTab op, PhysW k,
-    double inv_odt, const double* __restrict__ S, const double* __restrict__ qref, const W* __restrict__ Dinv,
-    const double* __restrict__ rs, const double* __restrict__ cs, double* __restrict__ werr) {
+    double inv_odt, const double* __restrict__ src, const double* __restrict__ S, const double* __restrict__ qref,
+    const W* __restrict__ Dinv, const double* __restrict__ rs, const double* __restrict__ cs,
+    double* __restrict__ werr) {
   constexpr int n1 = P + 1, N = n1 * n1, n = 4 * N, EPB = FusedEPB<P>::value, FP = 4 * n1;
   extern __shared__ __align__(128) unsigned char dsm[];
   __shared__ __align__(8) unsigned long long mbar;
@@ -299,7 +300,8 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
     for (int v = 0; v < 4; ++v) {
       qq[v] = __ldg(qin + v * plane + gi);
       if (qref) qo[v] = __ldg(qref + v * plane + gi);
-      if (S) Sv[v] = -__ldg(S + v * plane + gi);
+      if (src) Sv[v] = __ldg(src + v * plane + gi);
+      if (S) Sv[v] -= __ldg(S + v * plane + gi);
     }
 #pragma unroll
     for (int c = 0; c < 5; ++c) mt[c] = met[c * plane + gi];
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
       acc.add_prod(sgR[i], sJ[le][1][v][j]);
       acc.add_prod(sgL[j], sJ[le][0][v][i]);
       acc.add_prod(sgR[j], sJ[le][2][v][i]);
-      // -acc / |J| - qc / (omega dt) - S
+      // -acc / |J| - qc / (omega dt) + src - S
       const dw F = dot2_add(acc.value(), ninvJ, qc[v], nodt, dw_from_double(Sv[v]));
       const int row = v * N + t;
       sr[le][row] = scaled_in_dw<W>(F, ok ? srs[le * n + row] : rs[(size_t)e * n + row]);
@@ -443,10 +445,10 @@ static void fused_launch(const Ctx& c, const LevelDev& L, const double* qin, dou
       c.E, qin, qout, L.met, L.face, nbr, L.op, c.ph, c.phw, inv_odt, src, S, qref, (const WT*)L.Dinv, L.rs, \
       L.cs, c.d_scal + 1)
   const bool dwf = flux_dw_sweep(c);
-  if (dwf && c.ph.p_ref != 0.0 && !src) {   // gauge storage: the double-word sweep
+  if (dwf && c.ph.p_ref != 0.0) {   // gauge storage: the double-word sweep
 #define PMG_FUSED_DW(WT)                                                                         \
   fused_sweep_dw_kernel<P, WT><<<blocks, threads, fused_smem<P, WT>(), s>>>(                       \
-      c.E, qin, qout, L.metW, L.faceW, nbr, L.opw, L.op, c.phw, inv_odt, S, qref,                  \
+      c.E, qin, qout, L.metW, L.faceW, nbr, L.opw, L.op, c.phw, inv_odt, src, S, qref,             \
       (const WT*)L.Dinv, L.rs, L.cs, c.d_scal + 1)
     if (prec == PMG_PREC_FP64) PMG_FUSED_DW(double);
     else if (prec == PMG_PREC_BF16R) PMG_FUSED_DW(__nv_bfloat16);
