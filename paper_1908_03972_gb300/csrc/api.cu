@@ -445,11 +445,13 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
     // 20.3 / 20.0 at 1024, 24.4 / 24.1 / 25.9 at 2304 and 27.6 / 29.4 / 36.5 at
     // 3136; with a P = 2 finest level, fused against split, ten P{2-1-0}
     // V-cycles take 4.71 / 4.88 ms at 64 and 5.36 / 5.50 at 1600 elements in
-    // double-word, 8.28 / 8.50 at 64 in binary64.  PMG_FUSE_MAX_P sets the highest fused P instead (-1: none).
+    // double-word, 8.28 / 8.50 at 64 in binary64.  A finest P = 0 level keeps to
+    // the limit of P = 1.  PMG_FUSE_MAX_P sets the highest fused P instead (-1:
+    // none).
     bool boundary = false;
     for (const FaceRec& fr : c.mesh.faces) boundary = boundary || fr.eR < 0;
     const bool words = flux_dw_sweep(c) && c.ph.p_ref != 0.0;
-    const int per_sm[3] = {1 << 20, words ? 36 : 16, words ? 16 : 8};
+    const int small1 = words ? 36 : 16, per_sm[3] = {l == 0 ? small1 : 1 << 20, small1, words ? 16 : 8};
     bool fuse = L.P <= 2 && c.E <= (long long)per_sm[L.P <= 2 ? L.P : 2] * n_sms;
     bool fuse3 = fused3_applies(L.P, c.E, n_sms);
     if (const char* env = getenv("PMG_FUSE_MAX_P")) {
