@@ -636,11 +636,11 @@ struct ProfScope {
 };
 
 // Level system residual F_l(q_l) - S_l into lev[l].F (norm into d_scal[0] if asked).
-static void system_residual(Ctx& c, int l, bool norm) {
+static void system_residual(Ctx& c, int l, bool norm, bool have_grad = false) {
   LevelDev& L = c.lev[l];
   {
     ProfScope ps(c, K_FACE, l);
-    launch_face_flux(c, L, L.q, c.stream);
+    launch_face_flux(c, L, L.q, c.stream, false, have_grad);
   }
   {
     ProfScope ps(c, K_VOLUME, l);
@@ -711,20 +711,24 @@ static int sweeps(Ctx& c, int l, int n, bool F_valid, bool final_residual, bool 
     if (final_residual) system_residual(c, l, final_norm);
     return swaps;
   }
+  // viscous: each update also leaves the broken gradients of its result (have_grad) for the next face launch
+  bool have_grad = false;
   for (; s < n; ++s) {
     {
       ProfScope ps(c, K_FACE, l);
-      launch_face_flux(c, L, L.q, c.stream, true);
+      launch_face_flux(c, L, L.q, c.stream, true, have_grad);
     }
     {
       ProfScope ps(c, K_VOLUME, l);
       if (volume_dw_applies(c))
         launch_volume_apply_dw(c, L, L.q, 1.0 / c.omega_dt, src, S, qref, c.cfg.block_prec, c.stream);
       else
-        launch_volume_apply(c, L, L.q, 1.0 / c.omega_dt, src, S, qref, c.cfg.block_prec, c.stream);
+        launch_volume_apply(c, L, L.q, 1.0 / c.omega_dt, src, S, qref, c.cfg.block_prec, c.stream,
+                            s + 1 < n || final_residual);
     }
+    have_grad = c.ph.mu > 0.0;
   }
-  if (final_residual) system_residual(c, l, final_norm);
+  if (final_residual) system_residual(c, l, final_norm, have_grad);
   return 0;
 }
 

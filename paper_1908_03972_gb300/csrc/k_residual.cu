@@ -206,8 +206,9 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
                                                      const W* __restrict__ Dinv, const double* __restrict__ rs,
                                                      const double* __restrict__ cs,
                                                      const double* __restrict__ Qj, const double* __restrict__ Gb,
-                                                     double* __restrict__ werr) {
+                                                     double* __restrict__ werr, double* Gnext) {
   constexpr int n1 = P + 1, N = n1 * n1, EPB = ElemsPerBlock<P>::value, n = 4 * N;
+  constexpr bool kGrad = APPLY && VISC && P > 0;   // Gnext: leave the broken gradients of the updated state
   using PF = VolPrefetch<P, W>;
   extern __shared__ __align__(128) unsigned char dsm[];
   __shared__ __align__(8) unsigned long long mbar[2];   // 0: face fluxes, 1: blocks and scales
@@ -216,6 +217,7 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
   __shared__ double sFt[EPB][4][N];
   __shared__ double sGt[EPB][4][N];
   __shared__ double sD[n1][n1], sgL[n1], sgR[n1];   // Dt, gL, gR
+  __shared__ double sDg[kGrad ? n1 : 1][kGrad ? n1 : 1];   // D
   __shared__ double sred[256 / 32];
 
   const int le = threadIdx.x / N, pt = threadIdx.x - le * N;
@@ -254,7 +256,10 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
       if (S) Sv[v] = __ldg(S + v * plane + g0);
     }
   }
-  if (threadIdx.x < n1 * n1) sD[threadIdx.x / n1][threadIdx.x % n1] = op.Dt[threadIdx.x / n1][threadIdx.x % n1];
+  if (threadIdx.x < n1 * n1) {
+    sD[threadIdx.x / n1][threadIdx.x % n1] = op.Dt[threadIdx.x / n1][threadIdx.x % n1];
+    if (kGrad) sDg[kGrad ? threadIdx.x / n1 : 0][kGrad ? threadIdx.x % n1 : 0] = op.D[threadIdx.x / n1][threadIdx.x % n1];
+  }
   if (threadIdx.x < n1) {
     sgL[threadIdx.x] = op.gL[threadIdx.x];
     sgR[threadIdx.x] = op.gR[threadIdx.x];
@@ -410,7 +415,37 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
         const int v = row / N, p2 = row - v * N;
         const size_t o = v * plane + (size_t)e * N + p2;
         const double csc = okS ? scs[le * n + row] : cs[(size_t)e * n + row];
-        qw[o] = q[o] + scaled_out<W>(acc[m], csc);
+        const double qv = q[o] + scaled_out<W>(acc[m], csc);
+        qw[o] = qv;
+        if (kGrad && Gnext) sFt[le][v][p2] = qv;
+      }
+    }
+    if (kGrad && Gnext) {
+      // The operations of grad_kernel (k_viscous.cu) on the updated state, which
+      // is here already: 16384 elements, sweep of P = 4 (BF16) 244 us with its
+      // gradient launch, 230 without; P = 2 71 and 69, P = 1 30.7 and 28.5,
+      // a launch gap less each.
+      __syncthreads();
+      if (active) {
+#pragma unroll
+        for (int v = 0; v < 3; ++v) sGt[le][v][pt] = sFt[le][v + 1][pt] - sFt[le][v + 1][0];
+      }
+      __syncthreads();
+      if (active) {
+        const int i = pt % n1, j = pt / n1;
+        const double ia = invJ * __ldg(met + gi), ib = invJ * __ldg(met + plane + gi);
+        const double ic = invJ * __ldg(met + 2 * plane + gi), id = invJ * __ldg(met + 3 * plane + gi);
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+          double ax = 0.0, ae = 0.0;
+#pragma unroll
+          for (int m = 0; m < n1; ++m) {
+            ax = fma(sDg[kGrad ? i : 0][kGrad ? m : 0], sGt[le][v][j * n1 + m], ax);
+            ae = fma(sDg[kGrad ? j : 0][kGrad ? m : 0], sGt[le][v][m * n1 + i], ae);
+          }
+          Gnext[v * plane + gi] = fma(ia, ax, ic * ae);
+          Gnext[(3 + v) * plane + gi] = fma(ib, ax, id * ae);
+        }
       }
     }
   }
@@ -472,13 +507,13 @@ static int elems_per_block(int P) {
 
 int residual_blocks_for(int P, int E) { int epb = elems_per_block(P); return (E + epb - 1) / epb; }
 
-void launch_face_flux(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s, bool sweep) {
-  if (c.dim == 3) { launch_face_flux3(c, L, q, s); return; }
+void launch_face_flux(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s, bool sweep, bool have_grad) {
+  if (c.dim == 3) { launch_face_flux3(c, L, q, s, have_grad); return; }
   int total = c.n_faces * L.n1;
   // one warp per CTA: latency-bound threads, spread over every SM
   int threads = 32, blocks = (total + threads - 1) / threads;
   const bool visc = c.ph.mu > 0.0, dwf = sweep ? flux_dw_sweep(c) : flux_dw(c, L);
-  if (visc) launch_grad(c, L, q, s);
+  if (visc && !have_grad) launch_grad(c, L, q, s);
   const bool outdw = sweep && volume_dw_applies(c);
 #define PMG_FACE_V(PP, V, D, O)                                                                              \
   face_flux_kernel<PP, V, D, O><<<blocks, threads, 0, s>>>(c.d_faces, c.n_faces, c.E, q, L.face, L.faceW, L.Fcom, L.op, \
@@ -519,11 +554,11 @@ void launch_volume(const Ctx& c, const LevelDev& L, int level, const double* q, 
     if (c.ph.mu > 0.0)                                                                                       \
       volume_kernel<PP, double, false, true><<<blocks, threads, 0, s>>>(                                     \
           c.E, q, L.met, L.Fcom, L.op, c.ph, out, (int)mode, inv_odt, src, S, Sout, Pd, qn, partial, nullptr, \
-          nullptr, nullptr, nullptr, L.Qj, L.Gb, nullptr);                                                         \
+          nullptr, nullptr, nullptr, L.Qj, L.Gb, nullptr, nullptr);                                                         \
     else                                                                                                     \
       volume_kernel<PP, double, false, false><<<blocks, threads, 0, s>>>(                                    \
           c.E, q, L.met, L.Fcom, L.op, c.ph, out, (int)mode, inv_odt, src, S, Sout, Pd, qn, partial, nullptr, \
-          nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);                                             \
+          nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);                                             \
   } while (0)
   switch (L.P) {
     case 0: PMG_VOL(0); break;
@@ -538,7 +573,7 @@ void launch_volume(const Ctx& c, const LevelDev& L, int level, const double* q, 
 
 template <class W>
 static void volume_apply_dispatch(const Ctx& c, const LevelDev& L, double* q, double inv_odt, const double* src,
-                                  const double* S, const double* qn, cudaStream_t s) {
+                                  const double* S, const double* qn, double* gnext, cudaStream_t s) {
   int threads = residual_threads_per_block(L.P);
   int blocks = residual_blocks_for(L.P, c.E);
   const W* Dinv = (const W*)L.Dinv;
@@ -550,12 +585,12 @@ static void volume_apply_dispatch(const Ctx& c, const LevelDev& L, double* q, do
       volume_kernel<PP, W, true, true><<<blocks, threads, sm, s>>>(c.E, q, L.met, L.Fcom, L.op, c.ph, nullptr,  \
                                                                    (int)RES_SYSTEM, inv_odt, src, S, nullptr,   \
                                                                    nullptr, qn, nullptr, q, Dinv, L.rs, L.cs,   \
-                                                                   L.Qj, L.Gb, werr);                           \
+                                                                   L.Qj, L.Gb, werr, gnext);                    \
     else                                                                                                       \
       volume_kernel<PP, W, true, false><<<blocks, threads, sm, s>>>(c.E, q, L.met, L.Fcom, L.op, c.ph, nullptr, \
                                                                     (int)RES_SYSTEM, inv_odt, src, S, nullptr,  \
                                                                     nullptr, qn, nullptr, q, Dinv, L.rs, L.cs,  \
-                                                                    nullptr, nullptr, werr);                    \
+                                                                    nullptr, nullptr, werr, nullptr);           \
   } while (0)
   switch (L.P) {
     case 0: PMG_VA(0); break;
@@ -569,13 +604,15 @@ static void volume_apply_dispatch(const Ctx& c, const LevelDev& L, double* q, do
 }
 
 // Level-system residual of the current state followed, in the same launch,
-// by the element-Jacobi update of that state (after launch_face_flux).
+// by the element-Jacobi update of that state (after launch_face_flux).  With
+// grad_next (mu > 0) the broken gradients of the updated state are left in L.Gb.
 void launch_volume_apply(const Ctx& c, const LevelDev& L, double* q, double inv_odt, const double* src,
-                         const double* S, const double* qn, int prec, cudaStream_t s) {
-  if (c.dim == 3) { launch_volume_apply3(c, L, q, inv_odt, src, S, qn, prec, s); return; }
-  if (prec == PMG_PREC_FP64) volume_apply_dispatch<double>(c, L, q, inv_odt, src, S, qn, s);
-  else if (prec == PMG_PREC_BF16R) volume_apply_dispatch<__nv_bfloat16>(c, L, q, inv_odt, src, S, qn, s);
-  else volume_apply_dispatch<float>(c, L, q, inv_odt, src, S, qn, s);
+                         const double* S, const double* qn, int prec, cudaStream_t s, bool grad_next) {
+  double* gnext = grad_next && c.ph.mu > 0.0 && L.P > 0 ? L.Gb : nullptr;
+  if (c.dim == 3) { launch_volume_apply3(c, L, q, inv_odt, src, S, qn, gnext, prec, s); return; }
+  if (prec == PMG_PREC_FP64) volume_apply_dispatch<double>(c, L, q, inv_odt, src, S, qn, gnext, s);
+  else if (prec == PMG_PREC_BF16R) volume_apply_dispatch<__nv_bfloat16>(c, L, q, inv_odt, src, S, qn, gnext, s);
+  else volume_apply_dispatch<float>(c, L, q, inv_odt, src, S, qn, gnext, s);
 }
 
 // Dynamic shared memory limits of the fused residual-and-update kernels of

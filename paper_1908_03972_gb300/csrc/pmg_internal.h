@@ -264,7 +264,8 @@ inline bool flux_dw_sweep(const Ctx& c) { return c.cfg.flux_prec != PMG_FLUX_FP6
 // ---------------------------------------------------------- kernel launchers
 // sweep: the flux of an element-Jacobi sweep (flux_dw_sweep) rather than of
 // a residual evaluation (flux_dw)
-void launch_face_flux(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s, bool sweep = false);
+void launch_face_flux(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s, bool sweep = false,
+                      bool have_grad = false);
 cudaError_t prepare_residual_kernels(const Ctx& c);   // once per mesh upload
 // Residual-and-update sweep in double-word arithmetic (k_volume_dw.cu):
 // used where volume_dw_applies().
@@ -277,7 +278,7 @@ void launch_volume(const Ctx& c, const LevelDev& L, int level, const double* q, 
                    double* partial, cudaStream_t s, const double* qn = nullptr);
 void launch_norm_final(const double* partial, int n, double* out, cudaStream_t s);
 void launch_volume_apply(const Ctx& c, const LevelDev& L, double* q, double inv_odt, const double* src,
-                         const double* S, const double* qn, int prec, cudaStream_t s);
+                         const double* S, const double* qn, int prec, cudaStream_t s, bool grad_next);
 void launch_assemble(const Ctx& c, const LevelDev& L, const double* q, const double* d_dtau, double inv_odt,
                      cudaStream_t s);
 cudaError_t prepare_assemble(const Ctx& c);
@@ -309,12 +310,12 @@ void launch_loop_controller(LoopState* st, const double* scal, int* sing_flag, d
                             cudaGraphConditionalHandle h_refresh, cudaGraphConditionalHandle h_plain,
                             cudaStream_t s);
 // Hexahedral kernels (k3_*.cu); the launchers above dispatch to them when dim = 3.
-void launch_face_flux3(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s);
+void launch_face_flux3(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s, bool have_grad);
 void launch_volume3(const Ctx& c, const LevelDev& L, const double* q, double* out, ResMode mode, double inv_odt,
                     const double* src, const double* S, double* Sout, const double* Pd, double* partial,
                     cudaStream_t s, const double* qn);
 void launch_volume_apply3(const Ctx& c, const LevelDev& L, double* q, double inv_odt, const double* src,
-                          const double* S, const double* qn, int prec, cudaStream_t s);
+                          const double* S, const double* qn, double* gnext, int prec, cudaStream_t s);
 int residual_blocks_for3(int P, int E);
 // broken gradients of the viscous terms on hexahedra (Gb, 12 planes)
 void launch_grad3(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s);
