@@ -7,10 +7,10 @@
 // flight are what a thread can hold (ten), which leaves HBM half idle at
 // n = 320; here KC columns of each element at a time go through a ring of S
 // stages in shared memory with 16-byte asynchronous copies.  The columns are
-// used in the order of the plain loop, so the sums are the same bit for bit.
+// used in the order of the register loop (kept for inverses that L2 holds), so
+// the sums are the same bit for bit.
 // Measured on one GB300, FP32, us (before, columns in registers): 960 elements of
-// n = 320 97.6 -> 68.4 (393 MB, 5.7 TB/s), of n = 135 37.1 -> 28.3; 2304 of
-// n = 135 42.9 -> 37.6, of n = 40 12.9 -> 8.2.  Inside the residual-and-update
+// n = 320 97.6 -> 68.4 (393 MB, 5.7 TB/s), 2304 of n = 135 42.9 -> 37.6.  Inside the residual-and-update
 // kernel (k3_residual.cu) the ring takes the shared memory that its resident
 // CTAs need (n = 320: 104 -> 158 us), so that keeps its columns in registers.
 // Assembly and factorisation: k_assemble.cu, k_factor.cu.
@@ -89,7 +89,7 @@ using Stream3 =
 template <class W, int P>
 constexpr size_t stream3_bytes() { return P == 0 ? 0 : Stream3<W, P>::bytes; }
 
-template <class W, int P>
+template <class W, int P, bool STREAM>
 __global__ void __launch_bounds__(64) apply3_kernel(int E, const W* __restrict__ Dinv, const double* __restrict__ rs,
                                                     const double* __restrict__ cs, const double* __restrict__ r,
                                                     double* __restrict__ x, int accumulate) {
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(64) apply3_kernel(int E, const W* __restrict__
   using Stream = Stream3<W, P>;
   extern __shared__ __align__(16) unsigned char ring[];
   const int e0 = blockIdx.x * EPB, ne = min(EPB, E - e0);
-  if (P > 0)
+  if (STREAM)
     for (int c = 0; c < kStages3 - 1; ++c) Stream::issue(ring, Dinv, E, e0, ne, c);
   __shared__ Acc sr[EPB][n];
   const int le = threadIdx.x / N, pt = threadIdx.x - le * N;
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(64) apply3_kernel(int E, const W* __restrict__
       sr[le][v * N + pt] = scaled_in<W>(r[v * plane + (size_t)e * N + pt], rs[(size_t)e * n + v * N + pt]);
   }
   Acc acc[5] = {0, 0, 0, 0, 0};
-  if (P > 0) {
+  if (STREAM) {
 #pragma unroll 1
     for (int c = 0; c < Stream::NC; ++c) {
       async_wait<kStages3 - 2>();
@@ -137,8 +137,8 @@ __global__ void __launch_bounds__(64) apply3_kernel(int E, const W* __restrict__
     __syncthreads();
     if (!active) return;
     const W* Dm = Dinv + (size_t)e * n * n + pt;
-#pragma unroll
-    for (int k = 0; k < (P == 0 ? n : 0); ++k) {
+#pragma unroll 10
+    for (int k = 0; k < n; ++k) {
       const Acc rr = sr[le][k];
 #pragma unroll
       for (int v = 0; v < 5; ++v) acc[v] = fma(blk_val(__ldg(Dm + (size_t)k * n + v * N)), rr, acc[v]);
@@ -153,13 +153,27 @@ __global__ void __launch_bounds__(64) apply3_kernel(int E, const W* __restrict__
   }
 }
 
+// The ring pays once the inverses do not stay in the 129 MB L2.  Applied again and
+// again, 73 MB (FP32, n = 135) take 26 us through registers and 38 through the
+// ring; 88 MB (FP32, n = 320) 44 to 86, as they happen to lie in L2, and 47; from
+// 106 MB on the ring is faster (FP64, n = 135 101 against 82, n = 320 208 against
+// 122).
+static bool streams(size_t bytes) { return bytes > (size_t)80000000; }
+
 template <class W>
 static void apply3_dispatch(const Ctx& c, const LevelDev& L, const double* r, double* x, int acc, cudaStream_t s) {
   const W* Dinv = (const W*)L.Dinv;
-  const int N = L.N;
-  const int epb = N == 1 ? ApplyEPB3<0>::value : N == 8 ? ApplyEPB3<1>::value : N == 27 ? ApplyEPB3<2>::value : ApplyEPB3<3>::value;
-  const int threads = (epb * N + 31) / 32 * 32, blocks = (c.E + epb - 1) / epb;
-#define PMG_AP3(PP) apply3_kernel<W, PP><<<blocks, threads, stream3_bytes<W, PP>(), s>>>(c.E, Dinv, L.rs, L.cs, r, x, acc)
+  const bool ring = streams(sizeof(W) * c.E * L.n * L.n);
+#define PMG_AP3(PP)                                                                                          \
+  do {                                                                                                       \
+    constexpr int N = (PP + 1) * (PP + 1) * (PP + 1), epb = ApplyEPB3<PP>::value;                            \
+    const int threads = (epb * N + 31) / 32 * 32, blocks = (c.E + epb - 1) / epb;                            \
+    if (PP > 0 && ring)                                                                                      \
+      apply3_kernel<W, PP, (PP > 0)>                                                                         \
+          <<<blocks, threads, stream3_bytes<W, PP>(), s>>>(c.E, Dinv, L.rs, L.cs, r, x, acc);                \
+    else                                                                                                     \
+      apply3_kernel<W, PP, false><<<blocks, threads, 0, s>>>(c.E, Dinv, L.rs, L.cs, r, x, acc);              \
+  } while (0)
   switch (L.P) {
     case 0: PMG_AP3(0); break;
     case 1: PMG_AP3(1); break;
@@ -175,9 +189,9 @@ static cudaError_t prepare3(int P) {
   constexpr cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   switch (P) {
     case 0: return cudaSuccess;
-    case 1: return cudaFuncSetAttribute(apply3_kernel<W, 1>, a, (int)stream3_bytes<W, 1>());
-    case 2: return cudaFuncSetAttribute(apply3_kernel<W, 2>, a, (int)stream3_bytes<W, 2>());
-    default: return cudaFuncSetAttribute(apply3_kernel<W, 3>, a, (int)stream3_bytes<W, 3>());
+    case 1: return cudaFuncSetAttribute(apply3_kernel<W, 1, true>, a, (int)stream3_bytes<W, 1>());
+    case 2: return cudaFuncSetAttribute(apply3_kernel<W, 2, true>, a, (int)stream3_bytes<W, 2>());
+    default: return cudaFuncSetAttribute(apply3_kernel<W, 3, true>, a, (int)stream3_bytes<W, 3>());
   }
 }
 cudaError_t prepare_apply3(const Ctx& c) {
