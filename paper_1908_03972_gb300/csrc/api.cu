@@ -386,8 +386,8 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
   PMG_CK(dalloc(&c.d_faces, fbuf.size()));
   PMG_CK(cudaMemcpy(c.d_faces, fbuf.data(), sizeof(int) * fbuf.size(), cudaMemcpyHostToDevice));
   size_t maxtot = 0;
-  int maxblocks = 1, n_sms = 0;
-  PMG_CK(cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, c.device));
+  int maxblocks = 1;
+  PMG_CK(cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, c.device));
   size_t wbytes = c.cfg.block_prec == PMG_PREC_FP64 ? 8 : c.cfg.block_prec == PMG_PREC_BF16R ? 2 : 4;
   for (int l = 0; l < c.cfg.n_levels; ++l) {
     LevelDev& L = c.lev[l];
@@ -452,8 +452,8 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
     for (const FaceRec& fr : c.mesh.faces) boundary = boundary || fr.eR < 0;
     const bool words = flux_dw_sweep(c) && c.ph.p_ref != 0.0;
     const int small1 = words ? 36 : 16, per_sm[3] = {l == 0 ? small1 : 1 << 20, small1, words ? 16 : 8};
-    bool fuse = L.P <= 2 && c.E <= (long long)per_sm[L.P <= 2 ? L.P : 2] * n_sms;
-    bool fuse3 = fused3_applies(L.P, c.E, n_sms);
+    bool fuse = L.P <= 2 && c.E <= (long long)per_sm[L.P <= 2 ? L.P : 2] * c.sms;
+    bool fuse3 = fused3_applies(L.P, c.E, c.sms);
     if (const char* env = getenv("PMG_FUSE_MAX_P")) {
       fuse = L.P <= atoi(env) && L.P <= 3;
       fuse3 = fuse3 && atoi(env) >= 0;

@@ -27,7 +27,7 @@
 // pivot_row[k] of the inverse).
 //
 // Layout by size: n <= 64 one warp per block (R = 2 rows a lane above 32), no
-// CTA barrier, in FP64 two warps at n = 64; 100 to 144 one CTA, a row per
+// CTA barrier, in FP64 two warps at n = 64 and for few blocks of 36 and 40; 100 to 144 one CTA, a row per
 // thread, in FP64 split over two column groups; n = 320 a cluster of 5 CTAs
 // (FP32, two clusters' CTAs per SM) or 4 (FP64), whose registers hold 64 or 80
 // columns of every row; the panel's owner writes its multipliers into every
@@ -588,7 +588,11 @@ cudaError_t reg_call(bool prepare, int E, const double* D, W* Dinv, double* rs, 
 
 // The block sizes 4 (P+1)^2 (quadrilaterals, P <= 5) and 5 (P+1)^3
 // (hexahedra, P <= 3).  FP64 elements are 64-bit registers: panels of 4 and
-// half the columns per thread from n = 100 on.
+// half the columns per thread from n = 100 on.  `few`: at most four blocks per
+// SM, where one block's latency is the time and two warps of one row a lane take
+// n = 36 from 154 to 101 us and n = 40 from 187 to 114; beyond, one warp of two
+// rows a lane issues less (1000 blocks of n = 40 in 285 against 335 us, 4096 of
+// n = 36 in 801 against 877).
 template <class W>
 cudaError_t reg_size32(bool prep, int n, int E, const double* D, W* Di, double* rs, double* cs, int* fl, int b,
                        cudaStream_t s) {
@@ -605,14 +609,18 @@ cudaError_t reg_size32(bool prep, int n, int E, const double* D, W* Di, double* 
     default: return reg_call<float, W, 320, 1, 1, 5, 8, 1, 2>(prep, E, D, Di, rs, cs, fl, b, s);
   }
 }
-cudaError_t reg_size64(bool prep, int n, int E, const double* D, double* Di, double* rs, double* cs, int* fl, int b,
-                       cudaStream_t s) {
+cudaError_t reg_size64(bool prep, int n, int E, bool few, const double* D, double* Di, double* rs, double* cs,
+                       int* fl, int b, cudaStream_t s) {
   switch (n) {
     case 4: return reg_call<double, double, 4, 1, 1, 1, 4, 4, 8>(prep, E, D, Di, rs, cs, fl, b, s);
     case 5: return reg_call<double, double, 5, 1, 1, 1, 4, 4, 8>(prep, E, D, Di, rs, cs, fl, b, s);
     case 16: return reg_call<double, double, 16, 1, 1, 1, 4, 4, 4>(prep, E, D, Di, rs, cs, fl, b, s);
-    case 36: return reg_call<double, double, 36, 2, 1, 1, 4, 4, 2>(prep, E, D, Di, rs, cs, fl, b, s);
-    case 40: return reg_call<double, double, 40, 2, 1, 1, 4, 4, 2>(prep, E, D, Di, rs, cs, fl, b, s);
+    case 36:
+      return few ? reg_call<double, double, 36, 1, 1, 1, 4, 1, 6>(prep, E, D, Di, rs, cs, fl, b, s)
+                 : reg_call<double, double, 36, 2, 1, 1, 4, 4, 2>(prep, E, D, Di, rs, cs, fl, b, s);
+    case 40:
+      return few ? reg_call<double, double, 40, 1, 1, 1, 4, 1, 6>(prep, E, D, Di, rs, cs, fl, b, s)
+                 : reg_call<double, double, 40, 2, 1, 1, 4, 4, 2>(prep, E, D, Di, rs, cs, fl, b, s);
     case 64: return reg_call<double, double, 64, 1, 1, 1, 4, 1, 5>(prep, E, D, Di, rs, cs, fl, b, s);
     case 100: return reg_call<double, double, 100, 1, 2, 1, 4, 1, 1>(prep, E, D, Di, rs, cs, fl, b, s);
     case 135: return reg_call<double, double, 135, 1, 2, 1, 4, 1, 1>(prep, E, D, Di, rs, cs, fl, b, s);
@@ -621,9 +629,9 @@ cudaError_t reg_size64(bool prep, int n, int E, const double* D, double* Di, dou
   }
 }
 
-cudaError_t reg_prec(bool prep, int prec, int n, int E, const double* D, void* Di, double* rs, double* cs, int* fl,
-                     int b, cudaStream_t s) {
-  if (prec == PMG_PREC_FP64) return reg_size64(prep, n, E, D, (double*)Di, rs, cs, fl, b, s);
+cudaError_t reg_prec(bool prep, int prec, int n, int E, int sms, const double* D, void* Di, double* rs, double* cs,
+                     int* fl, int b, cudaStream_t s) {
+  if (prec == PMG_PREC_FP64) return reg_size64(prep, n, E, E <= 4 * sms, D, (double*)Di, rs, cs, fl, b, s);
   if (prec == PMG_PREC_BF16R) return reg_size32<__nv_bfloat16>(prep, n, E, D, (__nv_bfloat16*)Di, rs, cs, fl, b, s);
   return reg_size32<float>(prep, n, E, D, (float*)Di, rs, cs, fl, b, s);
 }
@@ -637,7 +645,7 @@ void launch_factor(const Ctx& c, LevelDev& L, int level, int prec, int* flag, cu
     launch_factor_cluster(c, L, level, prec, C, flag, s);
     return;
   }
-  reg_prec(false, prec, L.n, c.E, L.Dfull, L.Dinv, L.rs, L.cs, flag, base, s);
+  reg_prec(false, prec, L.n, c.E, c.sms, L.Dfull, L.Dinv, L.rs, L.cs, flag, base, s);
 }
 
 // Opt the kernels of every level into the shared memory they need (once,
@@ -646,8 +654,8 @@ cudaError_t prepare_kernels(const Ctx& c) {
   for (int l = 0; l < c.cfg.n_levels; ++l) {
     const int n = c.lev[l].n, C = factor_cluster_size(n, c.cfg.block_prec);
     const cudaError_t e = C > 0 ? prepare_factor_cluster(n, c.cfg.block_prec, C)
-                                : reg_prec(true, c.cfg.block_prec, n, c.E, nullptr, nullptr, nullptr, nullptr, nullptr,
-                                           0, nullptr);
+                                : reg_prec(true, c.cfg.block_prec, n, c.E, c.sms, nullptr, nullptr, nullptr, nullptr,
+                                           nullptr, 0, nullptr);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

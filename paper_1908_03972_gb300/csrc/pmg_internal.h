@@ -185,7 +185,7 @@ struct Ctx {
   Profiler prof;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  int device = 0;
+  int device = 0, sms = 0;   // sms: the device's SMs, read at pmg_upload_mesh
   Phys ph;
   PhysW phw;                   // double-word copies of the gas constants
   MeshHost mesh;
