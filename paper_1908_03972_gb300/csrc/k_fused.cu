@@ -1,15 +1,16 @@
-// k_fused.cu -- one element-Jacobi sweep of a coarse P-level in one launch.
+// k_fused.cu -- one element-Jacobi sweep of a small P-level in one launch (which
+// levels: pmg_upload_mesh, with the measurements).
 //
-// On the coarse levels (few points per element, 4096-16384 threads per launch)
-// the separate face-flux, volume and block-apply launches are each bound by
+// On small levels (few points per element, up to 16384 threads per launch) the separate face-flux, volume and block-apply launches are each bound by
 // the latency of one thread's FP64 chain, not by throughput.  This kernel
 // fuses a whole sweep q_next = q + D^-1 (F(q) - S) (Section 2.4, eq.
 // smoothing_element_jacobi, on the level system of Section 3) per element:
 //
 //  1. own state and contravariant fluxes to shared memory;
 //  2. the element's own 4 (P+1) face points: own and neighbour traces (the
-//     neighbour from the input state), preconditioned Roe flux.  Each face is evaluated by both of
-//     its elements: twice the face arithmetic, but no grid-wide dependency;
+//     neighbour from the input state), preconditioned Roe flux.  Each face is
+//     evaluated by both of its elements: twice the face arithmetic, but no
+//     grid-wide dependency;
 //  3. divergence of each line, Dt F + gL F_com(-1) + gR F_com(+1) (at P = 0
 //     Dt is zero: the face fluxes alone), level-system epilogue (F - S, stage term
 //     relative to q^b or q^n);

@@ -24,7 +24,8 @@
 // formed, the viscous launches add only the face corrections to the broken
 // gradient already written.  Full-size cylinder residual (16384 quadrilaterals,
 // P = 4, viscous; one GB300): gradient 62 -> 38 us, face flux 118 -> 106 us,
-// residual 215 -> 136 us.
+// residual 215 -> 110 us (136 before five elements filled a CTA's warps,
+// sweep_common.cuh).
 //
 // Viscous terms (mu > 0, Section 2.1 fluxes, Section 2.3 common viscous flux):
 // a gradient launch (k_viscous.cu) first forms the broken gradients of
@@ -33,8 +34,9 @@
 // eq. com_grad_q, evaluates the viscous flux at q_com (eq. com_q) and
 // subtracts it from the Roe flux; it also stores q_com - q_own for both
 // elements.  The volume launch forms the corrected gradient at each solution
-// point (derivative plus DG correction of those jumps) and subtracts the
-// viscous flux from the inviscid one before the divergence.
+// point (broken gradient plus DG correction of those jumps) and subtracts the
+// viscous flux from the inviscid one before the divergence.  A sweep's update
+// leaves the broken gradients of its result for the next face launch.
 #include "sweep_common.cuh"
 
 namespace pmg {
