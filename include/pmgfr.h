@@ -124,7 +124,8 @@ typedef struct {
                      solution of eq. com_q and the BR2 common gradient of
                      eq. com_grad_q (penalty eta_f = 4, the number of faces
                      of a quadrilateral) to the residual and to the element
-                     blocks.  The fused coarse sweep is not used then. */
+                     blocks.  The fused coarse sweeps of quadrilaterals are
+                     not used then. */
   double Pr;      /* Prandtl number of the heat flux K_j = -(mu Cp / Pr)
                      dT/dx_j (0.72 in the paper); read when mu > 0 */
   double res_scale[4]; /* reference scale of each equation (mass, x and y
@@ -295,8 +296,8 @@ pmg_status pmg_set_blocks(pmg_ctx* ctx, int level, const double* D, int on_devic
 /* Factor the assembled blocks of a level (or all, level = -1) in the
  * configured precision: power-of-two row/column equilibration, then
  * Gauss-Jordan elimination with partial pivoting to the explicit inverse,
- * one CTA per block, or a thread-block cluster of 2, 4 or 8 CTAs for blocks
- * one CTA's shared memory cannot hold (same arithmetic, same result).
+ * with the block in the registers of a few warps, a CTA or a thread-block
+ * cluster by its size (same arithmetic, same result).
  * Returns PMG_ESINGULAR, naming the element and level of the highest such
  * block (level-major order), if a pivot is not finite or not
  * above n eps of the working precision (the equilibrated rows have unit size

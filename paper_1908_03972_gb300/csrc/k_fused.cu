@@ -1,8 +1,9 @@
 // k_fused.cu -- one element-Jacobi sweep of a small P-level in one launch (which
 // levels: pmg_upload_mesh, with the measurements).
 //
-// On small levels (few points per element, up to 16384 threads per launch) the separate face-flux, volume and block-apply launches are each bound by
-// the latency of one thread's FP64 chain, not by throughput.  This kernel
+// On small levels (few points per element, up to 16384 threads per launch) the
+// separate face-flux and volume launches are each bound by the latency of one
+// thread's chain, not by throughput.  This kernel
 // fuses a whole sweep q_next = q + D^-1 (F(q) - S) (Section 2.4, eq.
 // smoothing_element_jacobi, on the level system of Section 3) per element:
 //
