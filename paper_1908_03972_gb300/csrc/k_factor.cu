@@ -541,6 +541,9 @@ __global__ void __launch_bounds__(Lay<T, N, R, G, CL, B>::NE* EPC, MINB)
             for (int q = 0; q < VN; ++q) a[r][j + q] = fma(-F[r][s], u[q], a[r][j + q]);
         }
     }
+    // One warp meets no barrier in the next panel before it writes U again, and
+    // its votes and shuffles order no memory.
+    if (NE == 32) __syncwarp();
   }
   // a last group whose final columns are all padding still owes their turns
   const int turns = max(0, min(C / B, Y::NP - gid * (C / B)));
