@@ -220,7 +220,7 @@ __device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_a
 template <int P, class W, bool APPLY, bool VISC>
 __global__ void __launch_bounds__(64) volume3_kernel(int E, const double* q, const double* __restrict__ met,
                                                      const double* __restrict__ Fcom, const double* __restrict__ Qj,
-                                                     const double* __restrict__ Gb,
+                                                     const double* Gb,
                                                      OpTab op, Phys ph,
                                                      double* __restrict__ out, int mode, double inv_odt,
                                                      const double* __restrict__ src, const double* __restrict__ S,
@@ -229,7 +229,10 @@ __global__ void __launch_bounds__(64) volume3_kernel(int E, const double* q, con
                                                      double* qw, const W* __restrict__ Dinv,
                                                      const double* __restrict__ rs, const double* __restrict__ cs,
                                                      double* Gnext) {
-  constexpr bool kGrad = APPLY && VISC && P > 0;   // Gnext: leave the broken gradients of the updated state
+  // Gnext: leave the broken gradients of the updated state.  It is Gb itself (a
+  // point's own entries, read before they are written), which is then neither
+  // restricted nor read as constant.
+  constexpr bool kGrad = APPLY && VISC && P > 0;
   constexpr int n1 = P + 1, N = n1 * n1 * n1, NF = n1 * n1, EPB = EPB3<P>::value, n = 5 * N;
   using Acc = typename Blk<W>::acc;
   __shared__ double sF[EPB][3][5][N];
@@ -278,7 +281,7 @@ __global__ void __launch_bounds__(64) volume3_kernel(int E, const double* q, con
       for (int c = 0; c < 3; ++c) ja[d][c] = __ldg(met + (3 * d + c) * plane + gi);
     if (VISC && P > 0)
 #pragma unroll
-      for (int c = 0; c < 12; ++c) g[c] = __ldg(Gb + c * plane + gi);
+      for (int c = 0; c < 12; ++c) g[c] = kGrad ? Gb[c * plane + gi] : __ldg(Gb + c * plane + gi);
   }
   if (VISC) {
     async_wait_all();

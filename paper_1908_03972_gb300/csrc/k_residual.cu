@@ -207,10 +207,13 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
                                                      double* __restrict__ partial, double* qw,
                                                      const W* __restrict__ Dinv, const double* __restrict__ rs,
                                                      const double* __restrict__ cs,
-                                                     const double* __restrict__ Qj, const double* __restrict__ Gb,
+                                                     const double* __restrict__ Qj, const double* Gb,
                                                      double* __restrict__ werr, double* Gnext) {
   constexpr int n1 = P + 1, N = n1 * n1, EPB = ElemsPerBlock<P>::value, n = 4 * N;
-  constexpr bool kGrad = APPLY && VISC && P > 0;   // Gnext: leave the broken gradients of the updated state
+  // Gnext: leave the broken gradients of the updated state.  It is Gb itself (a
+  // point's own entries, read before they are written), which is then neither
+  // restricted nor read as constant.
+  constexpr bool kGrad = APPLY && VISC && P > 0;
   using PF = VolPrefetch<P, W>;
   extern __shared__ __align__(128) unsigned char dsm[];
   __shared__ __align__(8) unsigned long long mbar[2];   // 0: face fluxes, 1: blocks and scales
@@ -293,8 +296,9 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
         const double* Qv = Qe + v * fplane;
         const double cx = fma(sgL[i], __ldg(Qv + 3 * n1 + j), sgR[i] * __ldg(Qv + 1 * n1 + j));
         const double ce = fma(sgL[j], __ldg(Qv + 0 * n1 + i), sgR[j] * __ldg(Qv + 2 * n1 + i));
-        gr[v] = fma(ia, cx, P > 0 ? fma(ic, ce, __ldg(Gb + v * plane + gi)) : ic * ce);
-        gr[3 + v] = fma(ib, cx, P > 0 ? fma(id, ce, __ldg(Gb + (3 + v) * plane + gi)) : id * ce);
+        const double *gx = Gb + v * plane + gi, *gy = Gb + (3 + v) * plane + gi;
+        gr[v] = fma(ia, cx, P > 0 ? fma(ic, ce, kGrad ? *gx : __ldg(gx)) : ic * ce);
+        gr[3 + v] = fma(ib, cx, P > 0 ? fma(id, ce, kGrad ? *gy : __ldg(gy)) : id * ce);
       }
       viscous_flux(qq[1], qq[2], gr, ph, fv, gv);
 #pragma unroll
