@@ -571,20 +571,26 @@ static cudaError_t copy_out(const Ctx& c, double* dst, const double* src, size_t
   return cudaStreamSynchronize(c.stream);
 }
 
-// Whether this context's kernels may read or write p themselves: memory of its
-// own device (a copy takes peers' memory too, a kernel only what is mapped).
-static bool own_memory(const Ctx& c, const void* p) {
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+// Whether this context's kernels may read or write the n doubles at p
+// themselves: memory of its own device from the first to the last byte, where a
+// double may lie.  A copy also takes peers' memory and any address, and refuses
+// a buffer that ends too early, where a kernel would fault.
+static bool own_memory(const Ctx& c, const void* p, size_t n) {
+  if (reinterpret_cast<uintptr_t>(p) % sizeof(double)) return false;
+  for (const char* b : {(const char*)p, (const char*)p + n * sizeof(double) - 1}) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, b) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (a.type != cudaMemoryTypeDevice || a.device != c.device) return false;
   }
-  return a.type == cudaMemoryTypeDevice && a.device == c.device;
+  return true;
 }
 
 // A caller's state into dst as the device holds it (pressure relative to p_gauge).
 static cudaError_t state_in(const Ctx& c, double* dst, const double* src, const LevelDev& L, int on_device) {
-  if (on_device && own_memory(c, src)) {
+  if (on_device && own_memory(c, src, L.tot)) {
     launch_copy_shift(L.tot / c.nv, L.tot, -c.ph.p_ref, src, dst, c.stream);
     return cudaGetLastError();
   }
@@ -1521,7 +1527,7 @@ pmg_status pmg_get_state(pmg_ctx* h, int level, double* q, int on_device) {
   pmg_status st = check_level(c, level);
   if (st) return st;
   const LevelDev& L = c.lev[level];
-  const bool direct = on_device && own_memory(c, q);
+  const bool direct = on_device && own_memory(c, q, L.tot);
   launch_copy_shift(L.tot / c.nv, L.tot, c.ph.p_ref, L.q, direct ? q : c.d_tmp0, c.stream);
   PMG_CK_LAUNCH();
   if (!direct) PMG_CK(copy_out(c, q, c.d_tmp0, L.tot, on_device));
