@@ -68,7 +68,10 @@ __device__ __forceinline__ double pow2_inv_scale_r(double m) {
   frexp(m, &ex);
   return ldexp(1.0, -ex);
 }
-__device__ __forceinline__ double pow2_d(int s) { return __longlong_as_double((long long)(s + 1023) << 52); }
+// 2^s, -1074 <= s <= 1024 (inf): rows up to the largest number have subnormal scales, 2^-1023 and 2^-1024
+__device__ __forceinline__ double pow2_d(int s) {
+  return __longlong_as_double(s > -1023 ? (long long)(s + 1023) << 52 : 1ll << (s + 1074));
+}
 __device__ __forceinline__ int pow2_exp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff) - 1023; }
 
 // d 2^s 2^t (applied in that order) in the working precision.
