@@ -52,7 +52,7 @@ __device__ __forceinline__ dw one_minus(dw x) { return dw{1.0f, 0.0f} - x; }
 // and dS the face area.  The pressure part is the one large term of the
 // momentum rows (p ~ 1/(gamma Ma^2) when the absolute pressure is stored);
 // the caller adds it.  The arrangement is roe_jump_d's (half the area in the
-// mass fluxes, one reciprocal for 1/T and 1/p) with sums of products
+// mass fluxes) with sums of products
 // renormalised once: about 1100 FP32 operations, 1400 as separate products and
 // sums.  64 elements (one GB300, launches of one warp's latency): the fused
 // P = 0 sweep 7.6 -> 5.6 us, the P = 1 face and update launches 5.2 -> 4.7 and
@@ -71,8 +71,7 @@ __device__ __forceinline__ void roe_flux_jump_dw(const dw qm[4], const dw qp[4],
   const dw u = qm[1] + half(du);
   const dw v = qm[2] + half(dv);
   const dw T = qm[3] + half(dT);
-  const dw r = rcp(p * T);
-  const dw iT = p * r, irho = T * (T * r), rho = p * iT;
+  const dw iT = rcp(T), irho = T * rcp(p), rho = p * iT;   // not through 1/(p T), which leaves the FP32 range first
   const dw c2 = k.gamma * T, ic2 = iT * k.inv_gamma;
   const dw vv = dot2(u, u, v, v);
   const dw e2 = min_dw(dw{1.0f, 0.0f}, max_dw(k.eps_min2, vv * ic2));
