@@ -73,7 +73,8 @@ typedef enum {
  * rounding, with the face traces, the jumps it takes and the central pressure
  * term in binary64; with gauge storage (p_gauge != 0) and mu = 0 the
  * residual-and-update of the element-Jacobi sweeps (the volume terms, the
- * level-system epilogue) is double-word too.  The sweeps are the smoother
+ * level-system epilogue) is double-word too, and in sweeps of one launch on
+ * P = 0 levels the pressure term.  The sweeps are the smoother
  * and the coarse levels only shape the FAS corrections of Section 3; the
  * finest level's residual defines the converged solution: the stopping
  * norm, the defect restricted to the coarse levels and pmg_residual. */

@@ -237,13 +237,15 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_kernel(
 }
 
 // The same sweep in double-word arithmetic (gauge storage, the sweeps of
-// PMG_FLUX_DW_SMOOTH): contravariant fluxes, face fluxes, the divergence and the level-system epilogue run on the FP32 pipes (dword.cuh;
-// see k_volume_dw.cu), while the traces and jumps the face flux takes are
-// still formed in binary64 relative to the element's first point.
+// PMG_FLUX_DW_SMOOTH): contravariant fluxes, face fluxes, the divergence and the
+// level-system epilogue run on the FP32 pipes (dword.cuh; see k_volume_dw.cu),
+// while the traces and jumps the face flux takes, relative to the element's first
+// point, and from P = 1 on its central pressure term are formed in binary64.
 template <int P, class W>
 __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
     int E, const double* __restrict__ qin, double* __restrict__ qout, const dw* __restrict__ met,
-    const dw* __restrict__ face, const int* __restrict__ nbr, OpTabW opw, OpTab op, PhysW k,
+    const dw* __restrict__ face, const double* __restrict__ face64, const int* __restrict__ nbr, OpTabW opw, OpTab op,
+    PhysW k,
     double inv_odt, const double* __restrict__ src, const double* __restrict__ S, const double* __restrict__ qref,
     const W* __restrict__ Dinv, const double* __restrict__ rs, const double* __restrict__ cs,
     double* __restrict__ werr) {
@@ -279,6 +281,7 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
   const int f = t / n1, kf = t - f * n1;
   double nq[4][n1], qq[4] = {0, 0, 0, 0}, qo[4] = {0, 0, 0, 0}, Sv[4] = {0, 0, 0, 0};
   dw gx = {}, gy = {}, gS = {}, mt[5] = {};
+  double g64[3] = {0, 0, 0};   // the face geometry of the pressure term (P > 0)
   int fn = 0;   // neighbour's face
   if (act) {
     const int en = __ldg(nbr + (e * 4 + f) * 3 + 0);
@@ -295,6 +298,9 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
     gx = g[0];
     gy = g[1];
     gS = g[2];
+    if (P > 0)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) g64[c] = __ldg(face64 + (((size_t)e * 4 + f) * n1 + kf) * 3 + c);
   }
   if (own) {
     const size_t gi = (size_t)e * N + t;
@@ -365,7 +371,7 @@ __global__ void __launch_bounds__(64, 1) fused_sweep_dw_kernel(
 #pragma unroll
     for (int v = 0; v < 4; ++v) dq[v] = P == 0 && (v == 0 || v == 3) ? sp[v] : sp[v] - sm[v];
     dw out[4];
-    face_roe_dw(ref[0], ref[3], sm, dq, gx, gy, gS, k, out);
+    face_roe_dw<(P > 0)>(ref[0], ref[3], sm, sp, dq, gx, gy, gS, g64, k, out);
 #pragma unroll
     for (int v = 0; v < 4; ++v) sJ[le][f][v][kf] = out[v];   // outward
   }
@@ -450,7 +456,7 @@ static void fused_launch(const Ctx& c, const LevelDev& L, const double* qin, dou
   if (dwf && c.ph.p_ref != 0.0) {   // gauge storage: the double-word sweep
 #define PMG_FUSED_DW(WT)                                                                         \
   fused_sweep_dw_kernel<P, WT><<<blocks, threads, fused_smem<P, WT>(), s>>>(                       \
-      c.E, qin, qout, L.metW, L.faceW, nbr, L.opw, L.op, c.phw, inv_odt, src, S, qref,             \
+      c.E, qin, qout, L.metW, L.faceW, L.face, nbr, L.opw, L.op, c.phw, inv_odt, src, S, qref,     \
       (const WT*)L.Dinv, L.rs, L.cs, c.d_scal + 1)
     if (prec == PMG_PREC_FP64) PMG_FUSED_DW(double);
     else if (prec == PMG_PREC_BF16R) PMG_FUSED_DW(__nv_bfloat16);

@@ -143,7 +143,8 @@ __global__ void __launch_bounds__(256) face_flux_kernel(const int* __restrict__ 
   if (OUTDW) {
     dw o[4];
     const dw* gw = faceW + (((size_t)eL * 4 + fL) * n1 + k) * 3;
-    face_roe_dw(ref[0], ref[3], sm, dq, gw[0], gw[1], gw[2], phw, o);
+    const double g64[3] = {nx, ny, dS};
+    face_roe_dw<true>(ref[0], ref[3], sm, sp, dq, gw[0], gw[1], gw[2], g64, phw, o);
     dw* Fw = reinterpret_cast<dw*>(Fcom);
 #pragma unroll
     for (int v = 0; v < 4; ++v) {

@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
     const int* __restrict__ toff, const int* __restrict__ tlayer, const int* __restrict__ telems,
     const int* __restrict__ tlnbr, int depth, int nsweep, int E, const double* __restrict__ qin,
     double* __restrict__ qout, const dw* __restrict__ met, const dw* __restrict__ face,
-    const int* __restrict__ nbr, OpTabW opw, OpTab op, PhysW k, double inv_odt,
+    const double* __restrict__ face64, const int* __restrict__ nbr, OpTabW opw, OpTab op, PhysW k, double inv_odt,
     const double* __restrict__ S, const double* __restrict__ qref, const W* __restrict__ Dinv,
     const double* __restrict__ rs, const double* __restrict__ cs) {
   using L = TileLayout<P, W>;
@@ -91,8 +91,12 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
   const bool mine = slot < M;
   const bool own = mine && tf < N;
   const int f = tf / n1, kf = tf - f * n1;
+  double g64[3] = {0, 0, 0};   // the face geometry of the pressure term (P > 0)
   if (mine) {
     const int e = telems[t0 + slot];
+    if (P > 0)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) g64[c] = __ldg(face64 + (((size_t)e * 4 + f) * n1 + kf) * 3 + c);
     const dw* g = face + (((size_t)e * 4 + f) * n1 + kf) * 3;
 #pragma unroll
     for (int c = 0; c < 3; ++c) sfg[((size_t)slot * FP + tf) * 3 + c] = g[c];
@@ -173,7 +177,7 @@ __global__ void __launch_bounds__(512, 1) tile_sweep_dw_kernel(
       for (int v = 0; v < 4; ++v) dq[v] = P == 0 && (v == 0 || v == 3) ? sp[v] : sp[v] - sm[v];
       const dw* g = sfg + ((size_t)slot * FP + tf) * 3;
       dw out[4];
-      face_roe_dw(ref[0], ref[3], sm, dq, g[0], g[1], g[2], k, out);
+      face_roe_dw<(P > 0)>(ref[0], ref[3], sm, sp, dq, g[0], g[1], g[2], g64, k, out);
 #pragma unroll
       for (int v = 0; v < 4; ++v) sJ[(((size_t)slot * 4 + f) * 4 + v) * n1 + kf] = out[v];   // outward
     }
@@ -257,7 +261,7 @@ static void tile_launch(const Ctx& c, const LevelDev& L, const double* qin, doub
   using Lay = TileLayout<P, W>;
   const int threads = (L.tile_M * Lay::FP + 31) / 32 * 32;
   tile_sweep_dw_kernel<P, W><<<L.n_tiles, threads, Lay::bytes(L.tile_M), s>>>(
-      L.d_toff, L.d_tlayer, L.d_telems, L.d_tlnbr, L.tile_depth, nsweep, c.E, qin, qout, L.metW, L.faceW,
+      L.d_toff, L.d_tlayer, L.d_telems, L.d_tlnbr, L.tile_depth, nsweep, c.E, qin, qout, L.metW, L.faceW, L.face,
       c.d_faces + 5 * c.n_faces, L.opw, L.op, c.phw, inv_odt, S, qref, (const W*)L.Dinv, L.rs, L.cs);
 }
 
