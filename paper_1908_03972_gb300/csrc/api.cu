@@ -490,10 +490,10 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
     PMG_CK(cudaMemset(L.S, 0, L.tot * 8));
     PMG_CK(cudaMemset(L.q, 0, L.tot * 8));
     {
-      // metrics and face geometry, and (2D) both in double-word for the
-      // sweeps, in one buffer and one copy
+      // metrics and face geometry, and both in double-word where the sweeps
+      // take them so, in one buffer and one copy
       const size_t nm = geo[l].met.size(), nfc = geo[l].face.size(), nb = nm + nfc;
-      const bool words = c.dim == 2;
+      const bool words = volume_dw_applies(c);
       std::vector<double> buf(words ? 2 * nb : nb);
       std::copy(geo[l].met.begin(), geo[l].met.end(), buf.begin());
       std::copy(geo[l].face.begin(), geo[l].face.end(), buf.begin() + nm);

@@ -122,7 +122,7 @@ struct LevelDev {
   double* Pd = nullptr;        // restricted defect (coarse levels)
   double* met = nullptr;       // 5 * E * N (2D), 10 * E * N (3D)
   double* face = nullptr;      // E * 4 * n1 * 3 (2D), E * 6 * NF * 4 (3D)
-  dw* metW = nullptr;          // the same in double-word, for the sweeps (2D)
+  dw* metW = nullptr;          // the same in double-word, where volume_dw_applies()
   dw* faceW = nullptr;
   double* Fcom = nullptr;      // nv * E * faces * NF common fluxes, outward
   // viscous terms (mu > 0 only); hexahedra in brackets
