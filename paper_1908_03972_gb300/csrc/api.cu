@@ -435,23 +435,26 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
         cudaMalloc(&L.Dinv, nn2 * wbytes) || dalloc(&L.rs, (size_t)c.E * L.n) || dalloc(&L.cs, (size_t)c.E * L.n))
       return fail(PMG_ENOMEM, "device allocation failed for level data");
     // Small levels are smoothed by a fused one-launch sweep (k_fused.cu; coarse
-    // P = 0 levels of hexahedra k3_fused.cu), which evaluates every face from both of its elements: the
-    // extra face work runs on SM sub-partitions the split launches leave idle and
-    // a launch is saved, until that work fills them.  The limits in elements per
-    // SM are where the two cross on 152 SMs: ten P{3-2-1-0} V-cycles with P = 0,
-    // P <= 1 and P <= 2 fused take, in double-word, 12.6 / 11.7 / 11.2 ms at 1024
-    // elements, 13.3 / 12.4 / 12.3 at 2304, 15.5 / 14.6 / 15.5 at 4096, 18.0 /
-    // 17.8 / 18.7 at 5184 and 20.0 / 20.0 / 21.2 at 6400; in binary64 21.0 /
-    // 20.3 / 20.0 at 1024, 24.4 / 24.1 / 25.9 at 2304 and 27.6 / 29.4 / 36.5 at
-    // 3136; with a P = 2 finest level, fused against split, ten P{2-1-0}
-    // V-cycles take 4.71 / 4.88 ms at 64 and 5.36 / 5.50 at 1600 elements in
-    // double-word, 8.28 / 8.50 at 64 in binary64.  A finest P = 0 level keeps to
-    // the limit of P = 1.  PMG_FUSE_MAX_P sets the highest fused P instead (-1:
-    // none).
+    // P = 0 levels of hexahedra k3_fused.cu), which evaluates every face from both
+    // of its elements: the extra face work runs on SM sub-partitions the split
+    // launches leave idle and a launch is saved, until that work fills them.  The
+    // limits in elements per SM are where the two cross on 152 SMs.  us a sweep,
+    // split / fused, 20 sweeps of one level (finest or coarse, the launches are the
+    // same), FP32 blocks (FP64 blocks cross at the same sizes):
+    //   double-word P = 2: 11.6 / 10.0 at 64 elements, 13.5 / 12.2 at 1936, 13.5 /
+    //     13.5 at 2304; P = 1: 10.0 / 8.5 at 64, 11.6 / 11.0 at 4096, 11.8 / 12.2 at
+    //     5184; P = 0: 8.5 / 6.7 at 64, 9.5 / 7.3 at 8100;
+    //   binary64 P = 2: 16.2 / 14.7 at 64, 17.9 / 16.2 at 1156, 18.4 / 21.5 at 1600;
+    //     P = 1: 15.3 / 13.6 at 64, 15.9 / 14.8 at 2304, 16.0 / 19.6 at 3136; P = 0:
+    //     13.6 / 10.7 at 64, 14.1 / 11.0 at 3136;
+    //   double-word faces in absolute pressure: the crossings of binary64 at P = 2
+    //     (15.4 / 14.7 at 1600, 15.9 / 16.5 at 1936) and P = 1 (13.5 / 13.5 at 3136).
+    // A finest P = 0 level keeps to the limit of P = 1.  PMG_FUSE_MAX_P sets the
+    // highest fused P instead (-1: none).
     bool boundary = false;
     for (const FaceRec& fr : c.mesh.faces) boundary = boundary || fr.eR < 0;
     const bool words = flux_dw_sweep(c) && c.ph.p_ref != 0.0;
-    const int small1 = words ? 36 : 16, per_sm[3] = {l == 0 ? small1 : 1 << 20, small1, words ? 16 : 8};
+    const int small1 = words ? 28 : 16, per_sm[3] = {l == 0 ? small1 : 1 << 20, small1, words ? 14 : 8};
     bool fuse = L.P <= 2 && c.E <= (long long)per_sm[L.P <= 2 ? L.P : 2] * c.sms;
     bool fuse3 = fused3_applies(L.P, c.E, c.sms);
     if (const char* env = getenv("PMG_FUSE_MAX_P")) {
