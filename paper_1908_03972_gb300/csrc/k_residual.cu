@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(256) face_flux_kernel(const int* __restrict__ 
 // face fluxes were formed from the old state by the preceding face launch,
 // and a CTA reads and writes only its own elements' states.  The update's
 // inputs are prefetched at entry (VolPrefetch, sweep_common.cuh).
-template <int P, class W, bool APPLY, bool VISC>
+template <int P, class W, bool APPLY, bool VISC, int EPB>
 __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
                                                      const double* __restrict__ met,
                                                      const double* __restrict__ Fcom, OpTab op, Phys ph,
@@ -210,12 +210,12 @@ __global__ void __launch_bounds__(256, 1) volume_kernel(int E, const double* q,
                                                      const double* __restrict__ cs,
                                                      const double* __restrict__ Qj, const double* Gb,
                                                      double* __restrict__ werr, double* Gnext) {
-  constexpr int n1 = P + 1, N = n1 * n1, EPB = ElemsPerBlock<P>::value, n = 4 * N;
+  constexpr int n1 = P + 1, N = n1 * n1, n = 4 * N;
   // Gnext: leave the broken gradients of the updated state.  It is Gb itself (a
   // point's own entries, read before they are written), which is then neither
   // restricted nor read as constant.
   constexpr bool kGrad = APPLY && VISC && P > 0;
-  using PF = VolPrefetch<P, W>;
+  using PF = VolPrefetch<P, W, EPB>;
   extern __shared__ __align__(128) unsigned char dsm[];
   __shared__ __align__(8) unsigned long long mbar[2];   // 0: face fluxes, 1: blocks and scales
   using Acc = typename Blk<W>::acc;
@@ -559,11 +559,11 @@ void launch_volume(const Ctx& c, const LevelDev& L, int level, const double* q, 
 #define PMG_VOL(PP)                                                                                          \
   do {                                                                                                       \
     if (c.ph.mu > 0.0)                                                                                       \
-      volume_kernel<PP, double, false, true><<<blocks, threads, 0, s>>>(                                     \
+      volume_kernel<PP, double, false, true, ElemsPerBlock<PP>::value><<<blocks, threads, 0, s>>>(                                     \
           c.E, q, L.met, L.Fcom, L.op, c.ph, out, (int)mode, inv_odt, src, S, Sout, Pd, qn, partial, nullptr, \
           nullptr, nullptr, nullptr, L.Qj, L.Gb, nullptr, nullptr);                                                         \
     else                                                                                                     \
-      volume_kernel<PP, double, false, false><<<blocks, threads, 0, s>>>(                                    \
+      volume_kernel<PP, double, false, false, ElemsPerBlock<PP>::value><<<blocks, threads, 0, s>>>(                                    \
           c.E, q, L.met, L.Fcom, L.op, c.ph, out, (int)mode, inv_odt, src, S, Sout, Pd, qn, partial, nullptr, \
           nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);                                             \
   } while (0)
@@ -581,24 +581,25 @@ void launch_volume(const Ctx& c, const LevelDev& L, int level, const double* q, 
 template <class W>
 static void volume_apply_dispatch(const Ctx& c, const LevelDev& L, double* q, double inv_odt, const double* src,
                                   const double* S, const double* qn, double* gnext, cudaStream_t s) {
-  int threads = residual_threads_per_block(L.P);
-  int blocks = residual_blocks_for(L.P, c.E);
   const W* Dinv = (const W*)L.Dinv;
   double* werr = c.d_scal + 1;
-#define PMG_VA(PP)                                                                                             \
+#define PMG_VA_E(PP, EP)                                                                                       \
   do {                                                                                                         \
-    const size_t sm = VolPrefetch<PP, W>::smem;                                                                \
+    constexpr int epb = EP<PP>::value, threads = elem_threads<PP, epb>();                                      \
+    const int blocks = (c.E + epb - 1) / epb;                                                                  \
+    const size_t sm = VolPrefetch<PP, W, epb>::smem;                                                           \
     if (c.ph.mu > 0.0)                                                                                         \
-      volume_kernel<PP, W, true, true><<<blocks, threads, sm, s>>>(c.E, q, L.met, L.Fcom, L.op, c.ph, nullptr,  \
-                                                                   (int)RES_SYSTEM, inv_odt, src, S, nullptr,   \
-                                                                   nullptr, qn, nullptr, q, Dinv, L.rs, L.cs,   \
-                                                                   L.Qj, L.Gb, werr, gnext);                    \
+      volume_kernel<PP, W, true, true, epb><<<blocks, threads, sm, s>>>(                                       \
+          c.E, q, L.met, L.Fcom, L.op, c.ph, nullptr, (int)RES_SYSTEM, inv_odt, src, S, nullptr, nullptr, qn,  \
+          nullptr, q, Dinv, L.rs, L.cs, L.Qj, L.Gb, werr, gnext);                                              \
     else                                                                                                       \
-      volume_kernel<PP, W, true, false><<<blocks, threads, sm, s>>>(c.E, q, L.met, L.Fcom, L.op, c.ph, nullptr, \
-                                                                    (int)RES_SYSTEM, inv_odt, src, S, nullptr,  \
-                                                                    nullptr, qn, nullptr, q, Dinv, L.rs, L.cs,  \
-                                                                    nullptr, nullptr, werr, nullptr);           \
+      volume_kernel<PP, W, true, false, epb><<<blocks, threads, sm, s>>>(                                      \
+          c.E, q, L.met, L.Fcom, L.op, c.ph, nullptr, (int)RES_SYSTEM, inv_odt, src, S, nullptr, nullptr, qn,  \
+          nullptr, q, Dinv, L.rs, L.cs, nullptr, nullptr, werr, nullptr);                                      \
   } while (0)
+#define PMG_VA(PP)                                                        \
+  if (few_elems(PP, c.E, c.sms)) PMG_VA_E(PP, FewElemsPerBlock);          \
+  else PMG_VA_E(PP, ElemsPerBlock)
   switch (L.P) {
     case 0: PMG_VA(0); break;
     case 1: PMG_VA(1); break;
@@ -608,6 +609,7 @@ static void volume_apply_dispatch(const Ctx& c, const LevelDev& L, double* q, do
     default: PMG_VA(5); break;
   }
 #undef PMG_VA
+#undef PMG_VA_E
 }
 
 // Level-system residual of the current state followed, in the same launch,
@@ -625,12 +627,17 @@ void launch_volume_apply(const Ctx& c, const LevelDev& L, double* q, double inv_
 // Dynamic shared memory limits of the fused residual-and-update kernels of
 // every level (their prefetch buffers can exceed the 48 KB default).
 template <class W>
-static cudaError_t prepare_apply(int P, bool visc) {
-#define PMG_PREP(PP)                                                                                          \
-  return visc ? cudaFuncSetAttribute(volume_kernel<PP, W, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                     (int)VolPrefetch<PP, W>::smem)                                            \
-              : cudaFuncSetAttribute(volume_kernel<PP, W, true, false>,                                        \
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)VolPrefetch<PP, W>::smem)
+static cudaError_t prepare_apply(int P, bool visc, bool few) {
+#define PMG_PREP_E(PP, EP)                                                                                    \
+  return visc ? cudaFuncSetAttribute(volume_kernel<PP, W, true, true, EP<PP>::value>,                          \
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,                              \
+                                     (int)VolPrefetch<PP, W, EP<PP>::value>::smem)                             \
+              : cudaFuncSetAttribute(volume_kernel<PP, W, true, false, EP<PP>::value>,                         \
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,                              \
+                                     (int)VolPrefetch<PP, W, EP<PP>::value>::smem)
+#define PMG_PREP(PP)                     \
+  if (few) PMG_PREP_E(PP, FewElemsPerBlock); \
+  PMG_PREP_E(PP, ElemsPerBlock)
   switch (P) {
     case 0: PMG_PREP(0);
     case 1: PMG_PREP(1);
@@ -640,14 +647,15 @@ static cudaError_t prepare_apply(int P, bool visc) {
     default: PMG_PREP(5);
   }
 #undef PMG_PREP
+#undef PMG_PREP_E
 }
 
 cudaError_t prepare_residual_kernels(const Ctx& c) {
   for (int l = 0; l < c.cfg.n_levels; ++l) {
-    const bool visc = c.ph.mu > 0.0;
-    cudaError_t e = c.cfg.block_prec == PMG_PREC_FP64    ? prepare_apply<double>(c.lev[l].P, visc)
-                    : c.cfg.block_prec == PMG_PREC_BF16R ? prepare_apply<__nv_bfloat16>(c.lev[l].P, visc)
-                                                         : prepare_apply<float>(c.lev[l].P, visc);
+    const bool visc = c.ph.mu > 0.0, few = few_elems(c.lev[l].P, c.E, c.sms);
+    cudaError_t e = c.cfg.block_prec == PMG_PREC_FP64    ? prepare_apply<double>(c.lev[l].P, visc, few)
+                    : c.cfg.block_prec == PMG_PREC_BF16R ? prepare_apply<__nv_bfloat16>(c.lev[l].P, visc, few)
+                                                         : prepare_apply<float>(c.lev[l].P, visc, few);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -25,14 +25,14 @@
 
 namespace pmg {
 
-template <int P, class W>
+template <int P, class W, int EPB>
 __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
     int E, double* q, const dw* __restrict__ met, const dw* __restrict__ Fcom, OpTabW opw, PhysW k,
     double inv_odt, const double* __restrict__ src, const double* __restrict__ S, const double* __restrict__ qref,
     const W* __restrict__ Dinv, const double* __restrict__ rs, const double* __restrict__ cs,
     double* __restrict__ werr) {
-  constexpr int n1 = P + 1, N = n1 * n1, EPB = ElemsPerBlock<P>::value, n = 4 * N;
-  using PF = VolPrefetch<P, W>;
+  constexpr int n1 = P + 1, N = n1 * n1, n = 4 * N;
+  using PF = VolPrefetch<P, W, EPB>;
   extern __shared__ __align__(128) unsigned char dsm[];
   __shared__ __align__(8) unsigned long long mbar[2];   // 0: face fluxes, 1: blocks and scales
   using Acc = typename Blk<W>::acc;
@@ -201,11 +201,17 @@ __global__ void __launch_bounds__(256, 1) volume_apply_dw_kernel(
 template <class W>
 static void dw_dispatch(const Ctx& c, const LevelDev& L, double* q, double inv_odt, const double* src,
                         const double* S, const double* qref, cudaStream_t s) {
-  const int threads = residual_threads_per_block(L.P), blocks = residual_blocks_for(L.P, c.E);
   const W* Dinv = (const W*)L.Dinv;
-#define PMG_VDW(PP)                                                                                         \
-  volume_apply_dw_kernel<PP, W><<<blocks, threads, VolPrefetch<PP, W>::smem, s>>>(                          \
-      c.E, q, L.metW, reinterpret_cast<const dw*>(L.Fcom), L.opw, c.phw, inv_odt, src, S, qref, Dinv, L.rs, L.cs, c.d_scal + 1)
+#define PMG_VDW_E(PP, EP)                                                                                   \
+  do {                                                                                                      \
+    constexpr int epb = EP<PP>::value, threads = elem_threads<PP, epb>();                                   \
+    volume_apply_dw_kernel<PP, W, epb><<<(c.E + epb - 1) / epb, threads, VolPrefetch<PP, W, epb>::smem, s>>>( \
+        c.E, q, L.metW, reinterpret_cast<const dw*>(L.Fcom), L.opw, c.phw, inv_odt, src, S, qref, Dinv, L.rs, \
+        L.cs, c.d_scal + 1);                                                                                \
+  } while (0)
+#define PMG_VDW(PP)                                                \
+  if (few_elems(PP, c.E, c.sms)) PMG_VDW_E(PP, FewElemsPerBlock);  \
+  else PMG_VDW_E(PP, ElemsPerBlock)
   switch (L.P) {
     case 0: PMG_VDW(0); break;
     case 1: PMG_VDW(1); break;
@@ -215,6 +221,7 @@ static void dw_dispatch(const Ctx& c, const LevelDev& L, double* q, double inv_o
     default: PMG_VDW(5); break;
   }
 #undef PMG_VDW
+#undef PMG_VDW_E
 }
 
 bool volume_dw_applies(const Ctx& c) {
@@ -229,10 +236,14 @@ void launch_volume_apply_dw(const Ctx& c, const LevelDev& L, double* q, double i
 }
 
 template <class W>
-static cudaError_t prep_dw(int P) {
-#define PMG_PDW(PP)                                                                                       \
-  return cudaFuncSetAttribute(volume_apply_dw_kernel<PP, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                              (int)VolPrefetch<PP, W>::smem)
+static cudaError_t prep_dw(int P, bool few) {
+#define PMG_PDW_E(PP, EP)                                                                                  \
+  return cudaFuncSetAttribute(volume_apply_dw_kernel<PP, W, EP<PP>::value>,                                \
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,                                 \
+                              (int)VolPrefetch<PP, W, EP<PP>::value>::smem)
+#define PMG_PDW(PP)                        \
+  if (few) PMG_PDW_E(PP, FewElemsPerBlock); \
+  PMG_PDW_E(PP, ElemsPerBlock)
   switch (P) {
     case 0: PMG_PDW(0);
     case 1: PMG_PDW(1);
@@ -242,13 +253,15 @@ static cudaError_t prep_dw(int P) {
     default: PMG_PDW(5);
   }
 #undef PMG_PDW
+#undef PMG_PDW_E
 }
 
 cudaError_t prepare_volume_dw_kernels(const Ctx& c) {
   for (int l = 0; l < c.cfg.n_levels; ++l) {
-    cudaError_t e = c.cfg.block_prec == PMG_PREC_FP64    ? prep_dw<double>(c.lev[l].P)
-                    : c.cfg.block_prec == PMG_PREC_BF16R ? prep_dw<__nv_bfloat16>(c.lev[l].P)
-                                                         : prep_dw<float>(c.lev[l].P);
+    const bool few = few_elems(c.lev[l].P, c.E, c.sms);
+    cudaError_t e = c.cfg.block_prec == PMG_PREC_FP64    ? prep_dw<double>(c.lev[l].P, few)
+                    : c.cfg.block_prec == PMG_PREC_BF16R ? prep_dw<__nv_bfloat16>(c.lev[l].P, few)
+                                                         : prep_dw<float>(c.lev[l].P, few);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -15,11 +15,24 @@ namespace pmg {
 // from 231 to 204, although the five inverses no longer fit the prefetch; at
 // P = 5 three (108 of 128; one filled 36 of 64) take 1073 elements from 16.2
 // to 12.5 us.
+// On few elements the updates are bound by the latency of their loads and chain
+// instead, and there they keep two and one (FewElemsPerBlock).  us a sweep, BF16
+// blocks, five / two: viscous P = 4 27.0 / 23.9 on 100 elements, 33.3 / 27.9 on
+// 784, 41.2 / 44.1 on 1600; inviscid double-word 15.4 / 14.1 and 17.6 / 15.3 on
+// the first two; P = 5 FP32, three / one: 17.8 / 16.6 on 100, 18.5 / 18.3 on 256,
+// and FP64 37.1 / 43.0 on 400.  The residual alone gains nothing from it.
 template <int P>
 struct ElemsPerBlock {
   static constexpr int N = (P + 1) * (P + 1);
   static constexpr int value = P == 0 ? 32 : P == 1 ? 8 : P == 2 ? 7 : P == 3 ? 4 : P == 4 ? 5 : 3;
 };
+template <int P>
+struct FewElemsPerBlock {
+  static constexpr int value = P == 4 ? 2 : P == 5 ? 1 : ElemsPerBlock<P>::value;
+};
+inline bool few_elems(int P, int E, int sms) { return P == 4 ? E <= 8 * sms : P == 5 && E <= sms; }
+template <int P, int EPB>
+constexpr int elem_threads() { return (EPB * (P + 1) * (P + 1) + 31) / 32 * 32; }
 
 // Prefetch layout of the residual-and-update sweep: the CTA's common face
 // fluxes, block scales and (where they fit, VolPrefetch::blocks) block
@@ -27,9 +40,9 @@ struct ElemsPerBlock {
 // entry, and the reference and forcing states are loaded into registers
 // there too: the latency of these reads then overlaps the flux arithmetic
 // instead of adding one L2 round trip per phase.
-template <int P, class W>
+template <int P, class W, int EPB>
 struct VolPrefetch {
-  static constexpr int n1 = P + 1, N = n1 * n1, EPB = ElemsPerBlock<P>::value, n = 4 * N;
+  static constexpr int n1 = P + 1, N = n1 * n1, n = 4 * N;
   static constexpr bool blocks = (size_t)EPB * n * n * sizeof(W) <= 40 * 1024;
   static constexpr size_t dinv_bytes = blocks ? (size_t)EPB * n * n * sizeof(W) : 0;
   static constexpr size_t scale_bytes = (size_t)EPB * n * sizeof(double);   // rs, then cs
