@@ -598,7 +598,7 @@ static void volume_apply_dispatch(const Ctx& c, const LevelDev& L, double* q, do
           nullptr, q, Dinv, L.rs, L.cs, nullptr, nullptr, werr, nullptr);                                      \
   } while (0)
 #define PMG_VA(PP)                                                        \
-  if (few_elems(PP, c.E, c.sms)) PMG_VA_E(PP, FewElemsPerBlock);          \
+  if (few_elems(PP, c.E, c.sms, c.cfg.block_prec, false)) PMG_VA_E(PP, FewElemsPerBlock); \
   else PMG_VA_E(PP, ElemsPerBlock)
   switch (L.P) {
     case 0: PMG_VA(0); break;
@@ -652,7 +652,7 @@ static cudaError_t prepare_apply(int P, bool visc, bool few) {
 
 cudaError_t prepare_residual_kernels(const Ctx& c) {
   for (int l = 0; l < c.cfg.n_levels; ++l) {
-    const bool visc = c.ph.mu > 0.0, few = few_elems(c.lev[l].P, c.E, c.sms);
+    const bool visc = c.ph.mu > 0.0, few = few_elems(c.lev[l].P, c.E, c.sms, c.cfg.block_prec, false);
     cudaError_t e = c.cfg.block_prec == PMG_PREC_FP64    ? prepare_apply<double>(c.lev[l].P, visc, few)
                     : c.cfg.block_prec == PMG_PREC_BF16R ? prepare_apply<__nv_bfloat16>(c.lev[l].P, visc, few)
                                                          : prepare_apply<float>(c.lev[l].P, visc, few);

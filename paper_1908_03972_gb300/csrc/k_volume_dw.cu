@@ -210,7 +210,7 @@ static void dw_dispatch(const Ctx& c, const LevelDev& L, double* q, double inv_o
         L.cs, c.d_scal + 1);                                                                                \
   } while (0)
 #define PMG_VDW(PP)                                                \
-  if (few_elems(PP, c.E, c.sms)) PMG_VDW_E(PP, FewElemsPerBlock);  \
+  if (few_elems(PP, c.E, c.sms, c.cfg.block_prec, true)) PMG_VDW_E(PP, FewElemsPerBlock); \
   else PMG_VDW_E(PP, ElemsPerBlock)
   switch (L.P) {
     case 0: PMG_VDW(0); break;
@@ -258,7 +258,7 @@ static cudaError_t prep_dw(int P, bool few) {
 
 cudaError_t prepare_volume_dw_kernels(const Ctx& c) {
   for (int l = 0; l < c.cfg.n_levels; ++l) {
-    const bool few = few_elems(c.lev[l].P, c.E, c.sms);
+    const bool few = few_elems(c.lev[l].P, c.E, c.sms, c.cfg.block_prec, true);
     cudaError_t e = c.cfg.block_prec == PMG_PREC_FP64    ? prep_dw<double>(c.lev[l].P, few)
                     : c.cfg.block_prec == PMG_PREC_BF16R ? prep_dw<__nv_bfloat16>(c.lev[l].P, few)
                                                          : prep_dw<float>(c.lev[l].P, few);

@@ -16,11 +16,16 @@ namespace pmg {
 // P = 5 three (108 of 128; one filled 36 of 64) take 1073 elements from 16.2
 // to 12.5 us.
 // On few elements the updates are bound by the latency of their loads and chain
-// instead, and there they keep two and one (FewElemsPerBlock).  us a sweep, BF16
-// blocks, five / two: viscous P = 4 27.0 / 23.9 on 100 elements, 33.3 / 27.9 on
-// 784, 41.2 / 44.1 on 1600; inviscid double-word 15.4 / 14.1 and 17.6 / 15.3 on
-// the first two; P = 5 FP32, three / one: 17.8 / 16.6 on 100, 18.5 / 18.3 on 256,
-// and FP64 37.1 / 43.0 on 400.  The residual alone gains nothing from it.
+// instead, and in double-word with FP32 or BF16 blocks, off the FP64 pipe, at any
+// size at P = 4: there they take two and one (FewElemsPerBlock).  us a sweep at
+// P = 4, five / two elements:
+//   binary64 viscous, BF16: 27.0 / 23.9 on 100 elements, 33.3 / 27.9 on 784, 41.2 /
+//     44.1 on 1600; FP32: 33.6 / 30.7 on 784, 59.2 / 54.3 on 2304, 102 / 106 on 4096;
+//   double-word, BF16: 15.4 / 14.1 on 100, 66.4 / 59.8 on 6400, 138 / 133 on 16384;
+//     FP32: 16.0 / 15.3, 79.4 / 76.2, 166 / 168; FP64: 28.5 / 28.3, 147 / 171.
+// P = 5, three / one: double-word FP32 17.8 / 16.6 on 100 elements, 19.5 / 19.1 on
+// 400, 21.4 / 20.9 on 784, BF16 20.4 / 21.1 there; binary64 FP32 24.0 / 22.9 on 100,
+// 24.8 / 25.8 on 400.  The residual alone gains nothing from it.
 template <int P>
 struct ElemsPerBlock {
   static constexpr int N = (P + 1) * (P + 1);
@@ -30,7 +35,11 @@ template <int P>
 struct FewElemsPerBlock {
   static constexpr int value = P == 4 ? 2 : P == 5 ? 1 : ElemsPerBlock<P>::value;
 };
-inline bool few_elems(int P, int E, int sms) { return P == 4 ? E <= 8 * sms : P == 5 && E <= sms; }
+inline bool few_elems(int P, int E, int sms, int prec, bool dword) {
+  const bool light = dword && prec != PMG_PREC_FP64;
+  if (P == 4) return light || E <= (prec == PMG_PREC_FP32 ? 20 : 8) * sms;
+  return P == 5 && E <= (light ? 4 : 1) * sms;
+}
 template <int P, int EPB>
 constexpr int elem_threads() { return (EPB * (P + 1) * (P + 1) + 31) / 32 * 32; }
 
