@@ -87,7 +87,7 @@ template <class W, int P>
 using Stream3 =
     BlockStream<W, 5 * (P + 1) * (P + 1) * (P + 1), ApplyEPB3<P>::value, StreamCols3<P>::value, kStages3>;
 template <class W, int P>
-constexpr size_t stream3_bytes() { return P == 0 ? 0 : Stream3<W, P>::bytes; }
+constexpr size_t stream3_bytes() { return P == 0 ? 0 : Stream3<W, P>::bytes; }   // P = 0 has no ring
 
 template <class W, int P, bool STREAM>
 __global__ void __launch_bounds__(64) apply3_kernel(int E, const W* __restrict__ Dinv, const double* __restrict__ rs,
@@ -153,23 +153,33 @@ __global__ void __launch_bounds__(64) apply3_kernel(int E, const W* __restrict__
   }
 }
 
-// The ring pays once the inverses do not stay in the 129 MB L2.  Applied again and
-// again, 73 MB (FP32, n = 135) take 26 us through registers and 38 through the
-// ring; 88 MB (FP32, n = 320) 44 to 86, as they happen to lie in L2, and 47; from
-// 106 MB on the ring is faster (FP64, n = 135 101 against 82, n = 320 208 against
-// 122).
-static bool streams(size_t bytes) { return bytes > (size_t)80000000; }
+// The ring pays where the inverses do not stay in the 129 MB L2 and its CTAs, whose
+// number on an SM the shared memory limits, run in one wave.  More waves cost FP64
+// inverses more than the ring gains, FP32 ones as much until n = 320 fills one and
+// a half; BF16 inverses, and those of n = 40 in FP32, win in any number.  Inverses
+// that L2 holds, applied again and again: 73 MB (FP32, n = 135) 37 us through the
+// ring and 34 through registers, 52 MB (FP64, n = 320) 120 and 86.  us from
+// memory, ring / registers (number of waves above one):
+//   FP64 n = 320: 124 / 215 (102 MB), 172 / 225 (597), 296 / 234 (819, 2), 529 / 491
+//     (1884, 4); n = 135: 94 / 114 (146), 184 / 131 (400, 2), 433 / 365 (1312, 5);
+//     n = 40: 59 / 57 (102, 2), 130 / 101 (346): never;
+//   FP32 n = 320: 56 / 108 (140), 126 / 134 (614), 147 / 139 (655, 2), 187 / 199
+//     (1065, 2), 271 / 304 (1638, 3); n = 135: 48 / 60 (126), 70 / 69 (219), 87 /
+//     75 (255, 2), 145 / 144 (656, 3); n = 40: 41 / 41 (88, 2), 58 / 62 (173, 3);
+//   BF16 n = 320: 56 / 97 (149), 167 / 220 (819, 2); n = 135: 46 / 57 (100), 99 /
+//     113 (328, 2); n = 40: 42 / 55 (86, 2).
+template <class W, int P>
+constexpr bool has_ring() { return P > 1 || (P == 1 && sizeof(W) < 8); }
 
 template <class W>
 static void apply3_dispatch(const Ctx& c, const LevelDev& L, const double* r, double* x, int acc, cudaStream_t s) {
   const W* Dinv = (const W*)L.Dinv;
-  const bool ring = streams(sizeof(W) * c.E * L.n * L.n);
 #define PMG_AP3(PP)                                                                                          \
   do {                                                                                                       \
     constexpr int N = (PP + 1) * (PP + 1) * (PP + 1), epb = ApplyEPB3<PP>::value;                            \
     const int threads = (epb * N + 31) / 32 * 32, blocks = (c.E + epb - 1) / epb;                            \
-    if (PP > 0 && ring)                                                                                      \
-      apply3_kernel<W, PP, (PP > 0)>                                                                         \
+    if (has_ring<W, PP>() && L.ring)                                                                         \
+      apply3_kernel<W, PP, has_ring<W, PP>()>                                                                \
           <<<blocks, threads, stream3_bytes<W, PP>(), s>>>(c.E, Dinv, L.rs, L.cs, r, x, acc);                \
     else                                                                                                     \
       apply3_kernel<W, PP, false><<<blocks, threads, 0, s>>>(c.E, Dinv, L.rs, L.cs, r, x, acc);              \
@@ -183,23 +193,37 @@ static void apply3_dispatch(const Ctx& c, const LevelDev& L, const double* r, do
 #undef PMG_AP3
 }
 
-// Ring of the apply kernels beyond the default shared memory.
+// Shared memory of the ring and whether a level's apply uses it (above).
+template <class W, int P>
+static cudaError_t prepare_ring(const Ctx& c, LevelDev& L) {
+  L.ring = false;
+  if (!has_ring<W, P>()) return cudaSuccess;
+  constexpr int N = (P + 1) * (P + 1) * (P + 1), epb = ApplyEPB3<P>::value;
+  auto* k = apply3_kernel<W, P, has_ring<W, P>()>;
+  constexpr size_t bytes = stream3_bytes<W, P>();
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  int resident = 0;
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k, (epb * N + 31) / 32 * 32, bytes);
+  const long long blocks = (c.E + epb - 1) / epb, wave = (long long)resident * c.sms;
+  const bool any = sizeof(W) == 2 || P == 1 || (sizeof(W) == 4 && P == 3 && 2 * blocks >= 3 * wave);
+  L.ring = sizeof(W) * c.E * L.n * L.n > (size_t)80000000 && (blocks <= wave || any);
+  return e;
+}
 template <class W>
-static cudaError_t prepare3(int P) {
-  constexpr cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  switch (P) {
-    case 0: return cudaSuccess;
-    case 1: return cudaFuncSetAttribute(apply3_kernel<W, 1, true>, a, (int)stream3_bytes<W, 1>());
-    case 2: return cudaFuncSetAttribute(apply3_kernel<W, 2, true>, a, (int)stream3_bytes<W, 2>());
-    default: return cudaFuncSetAttribute(apply3_kernel<W, 3, true>, a, (int)stream3_bytes<W, 3>());
+static cudaError_t prepare3(const Ctx& c, LevelDev& L) {
+  switch (L.P) {
+    case 0: return prepare_ring<W, 0>(c, L);
+    case 1: return prepare_ring<W, 1>(c, L);
+    case 2: return prepare_ring<W, 2>(c, L);
+    default: return prepare_ring<W, 3>(c, L);
   }
 }
-cudaError_t prepare_apply3(const Ctx& c) {
+cudaError_t prepare_apply3(Ctx& c) {
   for (int l = 0; l < c.cfg.n_levels; ++l) {
-    const int P = c.lev[l].P;
-    const cudaError_t e = c.cfg.block_prec == PMG_PREC_FP64    ? prepare3<double>(P)
-                          : c.cfg.block_prec == PMG_PREC_BF16R ? prepare3<__nv_bfloat16>(P)
-                                                               : prepare3<float>(P);
+    const cudaError_t e = c.cfg.block_prec == PMG_PREC_FP64    ? prepare3<double>(c, c.lev[l])
+                          : c.cfg.block_prec == PMG_PREC_BF16R ? prepare3<__nv_bfloat16>(c, c.lev[l])
+                                                               : prepare3<float>(c, c.lev[l]);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -133,6 +133,7 @@ struct LevelDev {
   double* fJinv = nullptr;     // E * 4 * n1 [E * 6 * NF]: 1/|J| at the face points
   double* Dfull = nullptr;     // E * n * n assembled FP64 blocks (row-major)
   void* Dinv = nullptr;        // E * n * n factored inverse (column-major), FP32 or FP64
+  bool ring = false;           // hexahedra: the block apply takes the inverses through its ring
   double* rs = nullptr;        // E * n row scales
   double* cs = nullptr;        // E * n column scales
   bool assembled = false, factored = false;
@@ -319,7 +320,7 @@ void launch_volume_apply3(const Ctx& c, const LevelDev& L, double* q, double inv
 int residual_blocks_for3(int P, int E);
 // broken gradients of the viscous terms on hexahedra (Gb, 12 planes)
 void launch_grad3(const Ctx& c, const LevelDev& L, const double* q, cudaStream_t s);
-cudaError_t prepare_apply3(const Ctx& c);
+cudaError_t prepare_apply3(Ctx& c);
 void launch_apply3(const Ctx& c, const LevelDev& L, int prec, const double* r, double* x, int accumulate,
                    cudaStream_t s);
 void launch_bsum_update3(const Ctx& c, int N, const double* qn, double* const* R, const double* b, int nr,
