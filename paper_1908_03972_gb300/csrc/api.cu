@@ -419,12 +419,7 @@ pmg_status pmg_upload_mesh(pmg_ctx* h, const pmg_mesh* m) {
     L.op.pen = 4.0 * 0.5 * L.n1 * L.n1;
     memset(&L.opw, 0, sizeof(L.opw));
     for (int i = 0; i < L.n1; ++i) {
-      for (int k = 0; k < L.n1; ++k) {
-        L.opw.D[i][k] = dw_const(L.op.D[i][k]);
-        L.opw.Dt[i][k] = dw_const(L.op.Dt[i][k]);
-      }
-      L.opw.lm[i] = dw_const(L.op.lm[i]);
-      L.opw.lp[i] = dw_const(L.op.lp[i]);
+      for (int k = 0; k < L.n1; ++k) L.opw.Dt[i][k] = dw_const(L.op.Dt[i][k]);
       L.opw.gL[i] = dw_const(L.op.gL[i]);
       L.opw.gR[i] = dw_const(L.op.gR[i]);
     }

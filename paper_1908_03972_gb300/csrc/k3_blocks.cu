@@ -15,7 +15,6 @@
 // CTAs need (n = 320: 104 -> 158 us), so that keeps its columns in registers.
 // Assembly and factorisation: k_assemble.cu, k_factor.cu.
 #include "pmg_internal.h"
-#include "physics3.cuh"
 
 namespace pmg {
 

@@ -15,7 +15,6 @@
 // 20.0 ms at 960 elements, 30.4 -> 28.2 at 1920, 67.1 -> 66.4 at 5760; of the
 // inviscid sphere 21.4 -> 20.1 ms at 2304 and equal at 6480.
 #include "pmg_internal.h"
-#include "physics3.cuh"
 
 namespace pmg {
 

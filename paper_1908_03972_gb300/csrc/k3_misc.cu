@@ -1,6 +1,5 @@
 // k3_misc.cu -- ESDIRK stage arithmetic (Section 2.4) on hexahedra, FP64.
 #include "pmg_internal.h"
-#include "physics3.cuh"
 
 namespace pmg {
 

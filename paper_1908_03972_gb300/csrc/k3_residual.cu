@@ -34,7 +34,6 @@
 // face geometry face[((e*6 + f)*NF + fp)*4] = (unit outward normal, area);
 // common fluxes Fcom[((v*E + e)*6 + f)*NF + fp], outward for element e.
 #include "pmg_internal.h"
-#include "physics3.cuh"
 
 namespace pmg {
 

@@ -37,7 +37,6 @@
 //   4096 quadrilaterals, P = 3         1.07 -> 0.27
 #include "pmg_internal.h"
 #include "physics_tan.cuh"
-#include "physics3.cuh"
 
 namespace pmg {
 

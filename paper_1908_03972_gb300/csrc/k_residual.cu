@@ -5,8 +5,11 @@
 //    neighbouring solution polynomials along the line normal to the face,
 //    evaluates the preconditioned Roe flux once and writes it, with opposite
 //    signs, into both elements' face slots (no atomics, exact conservation).
-//    On a boundary face the outer state is the ghost state of the boundary
-//    type (physics.cuh ghost_state), formed here relative to the reference.
+//    On a boundary face the outer state is the ghost state of the boundary type
+//    (the paper states no boundary treatment; reading: a ghost state enters the
+//    same common fluxes): the free stream at a far field, at walls the same p and
+//    T with the velocity's normal part (slip) or all of it (no-slip) reversed,
+//    formed here relative to the reference.
 //  * volume: one thread per solution point, several elements per CTA.
 //    Contravariant fluxes go to shared memory; a line's divergence is
 //    Dt F + gL F_com(-1) + gR F_com(+1), the derivative with the extrapolated

@@ -1,5 +1,5 @@
-// physics_dw.cuh -- the preconditioned Roe flux of physics.cuh (eq. invis_com,
-// same closed form, same order of operations) in double-word arithmetic
+// physics_dw.cuh -- the preconditioned Roe flux of physics.cuh (eq. invis_com, the
+// same closed form in the arrangement of roe_jump_d) in double-word arithmetic
 // (dword.cuh), for the residual kernels.  GB300's FP64 rate (2 lanes per
 // clock per SM) bounds the face-flux and sweep kernels; the same flux on the
 // FP32 pipes runs several times faster at ~2^-46 relative rounding.
@@ -15,7 +15,7 @@ namespace pmg {
 
 // Double-word copies of the gas constants (filled on the host).
 struct PhysW {
-  dw gamma, Cp, gm1, inv_gamma, inv_Cp, eps_min2;
+  dw gamma, Cp, inv_gamma, inv_Cp, eps_min2;
   dw p_ref;     // gauge reference pressure of the device states
   dw inv_gm1;   // 1 / (gamma - 1)
   double wait_ns;   // bound of the bulk-copy waits (< 0: give up at once)
@@ -23,16 +23,14 @@ struct PhysW {
 
 // Double-word copies of a level's 1D operators (see OpTab).
 struct OpTabW {
-  dw D[6][6];
   dw Dt[6][6];            // D - gL lm^T - gR lp^T
-  dw lm[6], lp[6], gL[6], gR[6];
+  dw gL[6], gR[6];
 };
 
 inline PhysW make_physw(const Phys& ph) {
   PhysW k;
   k.gamma = dw_const(ph.gamma);
   k.Cp = dw_const(ph.Cp);
-  k.gm1 = dw_const(ph.gm1);
   k.inv_gamma = dw_const(ph.inv_gamma);
   k.inv_Cp = dw_const(1.0 / ph.Cp);
   k.eps_min2 = dw_const(ph.eps_min * ph.eps_min);
@@ -46,7 +44,7 @@ inline PhysW make_physw(const Phys& ph) {
 __device__ __forceinline__ dw half(dw x) { return scale2(x, 0.5f); }
 __device__ __forceinline__ dw one_minus(dw x) { return dw{1.0f, 0.0f} - x; }
 
-// roe_flux_jump of physics.cuh in double-word, without the pressure part
+// roe_jump_d<2> of physics.cuh in double-word, without the pressure part
 // (pm^- + pm^+)/2 n dS of the central momentum flux: qm, qp hold absolute
 // pressure, dq = qp - qm (formed by the caller), (nx, ny) is the unit normal
 // and dS the face area.  The pressure part is the one large term of the
