@@ -50,12 +50,11 @@ __device__ __forceinline__ dw one_minus(dw x) { return dw{1.0f, 0.0f} - x; }
 // and dS the face area.  The pressure part is the one large term of the
 // momentum rows (p ~ 1/(gamma Ma^2) when the absolute pressure is stored);
 // the caller adds it.  The arrangement is roe_jump_d's (half the area in the
-// mass fluxes) with sums of products
-// renormalised once: about 1100 FP32 operations, 1400 as separate products and
-// sums.  64 elements (one GB300, launches of one warp's latency): the fused
-// P = 0 sweep 7.6 -> 5.6 us, the P = 1 face and update launches 5.2 -> 4.7 and
-// 6.4 -> 5.5 us, with the geometry kept in double-word and the states formed
-// on the FP32 pipes.
+// mass fluxes) with sums of products renormalised once: about 1100 FP32
+// operations, 1400 as separate products and sums.  64 elements (one GB300,
+// launches of one warp's latency): the fused P = 0 sweep 7.6 -> 5.4 us, the P = 1
+// face and update launches 5.2 -> 4.3 and 6.4 -> 4.7 us, with the geometry kept in
+// double-word and the states formed on the FP32 pipes.
 __device__ __forceinline__ void roe_flux_jump_dw(const dw qm[4], const dw qp[4], const dw dq[4], dw nx, dw ny,
                                                  dw dS, const PhysW& k, dw out[4]) {
   const dw h = half(dS);
