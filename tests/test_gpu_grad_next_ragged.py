@@ -1,9 +1,10 @@
 """Viscous sweeps whose update leaves the broken gradients for the next one, in
 place of those it read (k_residual.cu), against the oracle, on 121
-quadrilaterals: no number of elements that a CTA of the gradient, volume or
-update launches takes divides it, at any order, so the last CTA is part empty
-everywhere.  FP64 blocks and fluxes; the bound is that of the other V-cycle
-tests, 1e-8 of the change.
+quadrilaterals: no number of elements that a CTA of the gradient, residual or
+update launches takes divides it, so the last CTA is part empty (the updates of
+so few elements at P = 5 take one to a CTA; tests/test_gpu_few_elements.py has
+three).  FP64 blocks and fluxes; the bound is that of the other V-cycle tests,
+1e-8 of the change.
 """
 import numpy as np
 import pytest
